@@ -111,6 +111,7 @@ size_t carve_sorted(void* base, int64_t n_hits, int64_t n_events, int M, Sorted*
     Sorted o;
     o.coords = c.take<float4>(n_hits);
     o.phi = c.take<uint16_t>(n_hits);
+    o.bucket = c.take<uint16_t>(n_events * (M << kBucketBits));
     o.modoff = c.take<int32_t>(n_events * (M + 1));
     o.status = c.take<int32_t>(n_events);
     if (O) *O = o;
@@ -609,6 +610,7 @@ sbt_status sbt_reconstruct_host(sbt_handle* h, const float* x, const float* y, c
     auto chunk_views = [&](int c, Sorted& Oc, Staging& Sc) {
         const int64_t ev0 = e0[c];
         Oc = O;
+        Oc.bucket = O.bucket + ev0 * (h->C.M << kBucketBits);
         Oc.modoff = O.modoff + ev0 * (h->C.M + 1);
         Oc.status = O.status + ev0;
         Sc = S;

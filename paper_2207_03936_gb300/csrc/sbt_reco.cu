@@ -5,8 +5,9 @@
 //   1. k_sort: phi16 of every hit and its order by (module, phi16, input
 //      index) from one counting pass into (module, coarse phi) buckets and a
 //      sort inside each bucket, in shared memory (section "Sort by phi"); the
-//      sorted hits are written as AoS records (x, y, z, input index: float4,
-//      or fp16 x, y, z and a 16-bit index) + phi16;
+//      sorted hits are written as AoS records (x, y, z, phi16 and input
+//      index: float4, or fp16 x, y, z and a 16-bit index with phi16 beside),
+//      with the start of every bucket;
 //   2. k_search_*: for every module triplet (s, s+1, s+2): seeding over the unflagged
 //      middle hits, then following of every forming track to module s+3 with
 //      one-round claims on the hits, flags, and termination after two misses
@@ -78,27 +79,18 @@ __device__ __forceinline__ int phi_dist(uint32_t u, uint32_t v)
     return d1 < d2 ? d1 : d2;
 }
 
-// First position in phi[0, n) with phi >= v.
-__device__ __forceinline__ int lower_bound16(const uint16_t* phi, int n, uint32_t v)
+__device__ __forceinline__ float3 sub_rn(float4 a, float4 b)
 {
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if ((uint32_t)phi[mid] < v)
-            lo = mid + 1;
-        else
-            hi = mid;
-    }
-    return lo;
+    return make_float3(__fsub_rn(a.x, b.x), __fsub_rn(a.y, b.y), __fsub_rn(a.z, b.z));
 }
 
-// Straight-line extrapolation of (a, c) to the plane z = zt.
-__device__ __forceinline__ void extrapolate(float4 A, float4 Cc, float zt, float& xp, float& yp)
+// Straight-line extrapolation to the plane z = zt from the last hit c and its
+// difference d from the hit before it.
+__device__ __forceinline__ void extrapolate(float3 c, float3 d, float zt, float& xp, float& yp)
 {
-    float dz = __fsub_rn(Cc.z, A.z);
-    float tz = __fdiv_rn(__fsub_rn(zt, Cc.z), dz);
-    xp = __fadd_rn(Cc.x, __fmul_rn(__fsub_rn(Cc.x, A.x), tz));
-    yp = __fadd_rn(Cc.y, __fmul_rn(__fsub_rn(Cc.y, A.y), tz));
+    float tz = __fdiv_rn(__fsub_rn(zt, c.z), d.z);
+    xp = __fadd_rn(c.x, __fmul_rn(d.x, tz));
+    yp = __fadd_rn(c.y, __fmul_rn(d.y, tz));
 }
 
 __device__ __forceinline__ float scatter_of(float4 B, float xp, float yp)
@@ -152,8 +144,8 @@ __device__ __forceinline__ void fit_line(int n, Get get, float sigma, float* par
 // ------------------------------------------------------- shared layout ---
 
 enum Misc {
-    kErr = 0, kCnt0 = 1, kCnt1 = 2, kNFin = 3, kNTl = 4, kEvent = 5, kList = 6, kNOuter = 7,
-    kNew = 8, kWork = 9, kCMask = 10, kMiscN = 12
+    kErr = 0, kNFin = 1, kNTl = 2, kEvent = 3, kCMask = 4, kCnt0 = 5, kCnt1 = 6, kNew = 7, kWork = 8, kList = 9,
+    kNOuter = 10, kMiscN = 12
 };
 
 // Per-block shared memory of the search: flag bits, module offsets, counters,
@@ -202,19 +194,35 @@ __device__ inline Smem carve(unsigned char* raw, int nmax, int threads, int M)
 __device__ __forceinline__ bool flagged(const Smem& S, int p) { return (S.flag[p >> 5] >> (p & 31)) & 1u; }
 __device__ __forceinline__ void set_flag(const Smem& S, int p) { atomicOr(&S.flag[p >> 5], 1u << (p & 31)); }
 
-// Storage of the sorted hits.  HitsF32: float4 (x, y, z, input index as
-// int bits), 16 bytes.  HitsF16: x, y, z rounded to fp16 (nearest even) and
-// the input index in 16 bits, 8 bytes (the paper's fp16 AoS storage of hit
-// coordinates); every computation still runs in fp32, on the rounded values.
+// Storage of the sorted hits.  HitsF32: float4 (x, y, z, phi16 << 16 | input
+// index as int bits), 16 bytes: one load gives a window scan the key and the
+// position.  HitsF16: x, y, z rounded to fp16 (nearest even) and the input
+// index in 16 bits, 8 bytes (the paper's fp16 AoS storage of hit
+// coordinates), phi16 in an array of its own; every computation still runs in
+// fp32, on the rounded values.
 struct HitsF32 {
     using T = float4;
+    static constexpr bool kPhiArray = false;
     __device__ __forceinline__ static float round(float v) { return v; }
     __device__ __forceinline__ static float4 load(const T* p, int i) { return p[i]; }
-    __device__ __forceinline__ static void store(T* p, int64_t i, float4 c) { p[i] = c; }
+    __device__ __forceinline__ static void store(T* p, int64_t i, float4 c, uint32_t ph)
+    {
+        c.w = __int_as_float((int)(ph << 16) | __float_as_int(c.w));
+        p[i] = c;
+    }
+    __device__ __forceinline__ static uint32_t key(float4 c, const uint16_t*, int)
+    {
+        return (uint32_t)__float_as_int(c.w);
+    }
+    __device__ __forceinline__ static uint32_t phi_at(const T* p, const uint16_t*, int i)
+    {
+        return (uint32_t)__float_as_int(p[i].w) >> 16;
+    }
 };
 
 struct HitsF16 {
     using T = ushort4;
+    static constexpr bool kPhiArray = true;
     __device__ __forceinline__ static float round(float v) { return __half2float(__float2half_rn(v)); }
     __device__ __forceinline__ static float4 load(const T* p, int i)
     {
@@ -222,29 +230,44 @@ struct HitsF16 {
         return make_float4(__half2float(__ushort_as_half(u.x)), __half2float(__ushort_as_half(u.y)),
                            __half2float(__ushort_as_half(u.z)), __int_as_float((int)u.w));
     }
-    __device__ __forceinline__ static void store(T* p, int64_t i, float4 c)
+    __device__ __forceinline__ static void store(T* p, int64_t i, float4 c, uint32_t)
     {
         p[i] = make_ushort4(__half_as_ushort(__float2half_rn(c.x)), __half_as_ushort(__float2half_rn(c.y)),
                             __half_as_ushort(__float2half_rn(c.z)), (unsigned short)__float_as_int(c.w));
     }
+    __device__ __forceinline__ static uint32_t key(float4, const uint16_t* ph, int i) { return (uint32_t)ph[i] << 16; }
+    __device__ __forceinline__ static uint32_t phi_at(const T*, const uint16_t* ph, int i) { return ph[i]; }
 };
 
-// Sorted hits of one event, hit p as float4 (x, y, z, input index bits).
+// Event-local input index in a loaded record (below 2^14).
+__device__ __forceinline__ int index_of(float4 c) { return __float_as_int(c.w) & 0xFFFF; }
+
+// Sorted hits of one event: hit p as float4, its phi16.
 template <class HS>
 struct HitArr {
     const typename HS::T* p;
+    const uint16_t* ph;
     __device__ __forceinline__ float4 operator[](int i) const { return HS::load(p, i); }
+    // record and its phi16 << 16 | low bits
+    __device__ __forceinline__ float4 get(int i, uint32_t& key) const
+    {
+        const float4 c = HS::load(p, i);
+        key = HS::key(c, ph, i);
+        return c;
+    }
+    __device__ __forceinline__ uint32_t phi(int i) const { return HS::phi_at(p, ph, i); }
 };
 
 // What one event's search sees: its sorted hits (read-only) and its scratch.
 template <class HS>
 struct Region {
     HitArr<HS> coords;
-    const uint16_t* phi;
+    const uint16_t* bucket;     // first sorted position of each (module, phi16 >> 10)
     uint32_t* list;
     uint16_t* prev;
     unsigned long long* claim;  // the search's claim of sorted position p is claim[p & cmask]
     unsigned cmask;
+    unsigned long long* claim_all;  // by sorted position, for the tracklet filter
     unsigned long long* tracklets;
     uint32_t* tl_q;
     int lcap;
@@ -254,15 +277,16 @@ struct Region {
 };
 
 template <class HS>
-__device__ inline Region<HS> region_of(const Sorted& O, int off, const Work& W, int64_t hb, int64_t r,
-                                      int cap)
+__device__ inline Region<HS> region_of(const Sorted& O, int M, int e, int off, const Work& W, int64_t hb,
+                                      int64_t r, int cap)
 {
     Region<HS> R;
-    R.coords = HitArr<HS>{(const typename HS::T*)O.coords + off};
-    R.phi = O.phi + off;
+    R.coords = HitArr<HS>{(const typename HS::T*)O.coords + off, O.phi + off};
+    R.bucket = O.bucket + (int64_t)e * (M << kBucketBits);
     R.list = W.list + hb;
     R.prev = W.prev + hb;
-    R.claim = W.claim + hb;
+    R.claim_all = W.claim + hb;
+    R.claim = R.claim_all;
     R.cmask = ~0u;
     R.tracklets = W.tracklets + hb + r;
     R.tl_q = W.tl_q + hb + r;
@@ -308,7 +332,12 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* wsum, int* total
 // ------------------------------------------------------------- sorting ---
 
 constexpr int kSortThreads = 1024;
-constexpr int kSortBuckets = 4096;  // (module, top six bits of phi16)
+constexpr int kSortBuckets = kMaxModules << kBucketBits;  // (module, top bits of phi16)
+__device__ __forceinline__ int bucket_of(int m, uint32_t phi16)
+{
+    return (m << kBucketBits) | (int)(phi16 >> (16 - kBucketBits));
+}
+
 constexpr int kShortBucket = 32;    // buckets up to this size are sorted by one thread
 
 // Shared memory of the sort kernel: the bucketed entries phi16 << 14 | input
@@ -426,7 +455,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort(DevConfig C, Inputs in
             }
             const uint32_t ph = phi16_of(HS::round(xs[u]), HS::round(ys[u]));
             phi[i] = (uint16_t)ph;
-            atomicAdd(&cnt[(m << 6) | (int)(ph >> 10)], 1);
+            atomicAdd(&cnt[bucket_of(m, ph)], 1);
         }
     }
     __syncthreads();
@@ -458,7 +487,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort(DevConfig C, Inputs in
     for (int i = tid; i < n; i += NT) {
         const uint32_t ph = phi[i];
         const int m = in.module[off + i];
-        const int p = atomicAdd(&cnt[(m << 6) | (int)(ph >> 10)], 1);
+        const int p = atomicAdd(&cnt[bucket_of(m, ph)], 1);
         ent[p] = (ph << 14) | (uint32_t)i;
     }
     __syncthreads();
@@ -487,14 +516,18 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort(DevConfig C, Inputs in
         warp_bitonic(ent + lo, cnt[b] - lo);
     }
     for (int m = tid; m <= C.M; m += NT)
-        O.modoff[(int64_t)e * (C.M + 1) + m] = m == 0 ? 0 : (m < C.M ? cnt[(m << 6) - 1] : n);
+        O.modoff[(int64_t)e * (C.M + 1) + m] = m == 0 ? 0 : (m < C.M ? cnt[(m << kBucketBits) - 1] : n);
+    // bucket starts, two per store (the table has an even length)
+    uint32_t* const tab = (uint32_t*)(O.bucket + (int64_t)e * (C.M << kBucketBits));
+    for (int b = 2 * tid; b < C.M << kBucketBits; b += 2 * NT)
+        tab[b >> 1] = (uint32_t)(b > 0 ? cnt[b - 1] : 0) | ((uint32_t)cnt[b] << 16);
     __syncthreads();
     // phi16 by sorted position, and the sorted position of every input hit
     // (in the space of phi16 by input order, free now)
     uint16_t* rank = phi;
     for (int p = tid; p < n; p += NT) {
         const uint32_t en = ent[p];
-        O.phi[off + p] = (uint16_t)(en >> 14);
+        if (HS::kPhiArray) O.phi[off + p] = (uint16_t)(en >> 14);
         rank[en & 0x3FFFu] = (uint16_t)p;
     }
     __syncthreads();
@@ -513,7 +546,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort(DevConfig C, Inputs in
         }
 #pragma unroll
         for (int u = 0; u < 2; u++)
-            if (i0 + u * NT < n) HS::store((typename HS::T*)O.coords, (int64_t)off + q[u], c[u]);
+            if (i0 + u * NT < n) HS::store((typename HS::T*)O.coords, (int64_t)off + q[u], c[u], ent[q[u]] >> 14);
     }
     if (tid == 0) O.status[e] = SBT_OK;
 }
@@ -528,9 +561,9 @@ __device__ __forceinline__ uint32_t phi16_window(float x, float y)
     const float a7 = -0.0851330f, a9 = 0.0208351f;
     float ax = fabsf(x), ay = fabsf(y);
     float mx = fmaxf(ax, ay), mn = fminf(ax, ay);
-    float t = mx > 0.0f ? __fdividef(mn, mx) : 0.0f;
-    float t2 = t * t;
-    float p = ((((a9 * t2 + a7) * t2 + a5) * t2 + a3) * t2 + a1) * t;
+    const float t = mx > 0.0f ? __fdividef(mn, mx) : 0.0f;
+    const float t2 = t * t;
+    float p = __fmaf_rn(__fmaf_rn(__fmaf_rn(__fmaf_rn(a9, t2, a7), t2, a5), t2, a3), t2, a1) * t;
     if (ay > ax) p = 1.5707963f - p;
     if (x < 0.0f) p = 3.1415927f - p;
     if (y < 0.0f) p = -p;
@@ -547,7 +580,7 @@ __device__ __forceinline__ uint32_t phi16_window(float x, float y)
 __device__ __forceinline__ bool window_of(float xp, float yp, float cut, float sqrt_cut, uint32_t& lo,
                                           uint32_t& width)
 {
-    const float rp2 = xp * xp + yp * yp;
+    const float rp2 = __fmaf_rn(xp, xp, yp * yp);
     if (rp2 < 1.0e30f && rp2 > 4.0f * cut) {
         const float wf = sqrt_cut * rsqrtf(rp2 - cut) * (10430.378f * 1.0625f);
         if (wf < 16000.0f) {
@@ -583,41 +616,61 @@ struct PairGeo {
     __device__ __forceinline__ static bool on(int p, float x) { return (x < 0.0f) == (p != 0); }
 };
 
-// Visits the unflagged hits of plane `plane` of module [b0, b0 + nb) inside
-// the window that starts at sorted index lo_idx (all hits when not
-// windowed); the scatter of every visited hit is computed exactly (rounded
-// operations) and `better(sc, b)` orders candidates under the cut.
-template <class G, class Better, class Take, class HS>
-__device__ __forceinline__ void scan_from(const Smem& S, const Region<HS>& R, int b0, int nb, float xp,
-                                          float yp, float cut, bool windowed, int lo_idx,
-                                          uint32_t lo, uint32_t width, int plane, Better better,
-                                          Take take)
-{
-    for (int k = 0; k < nb; k++) {
-        int e = lo_idx + k;
-        if (e >= nb) e -= nb;
-        const int b = b0 + e;
-        // both loads issued together (b is inside the module either way)
-        const uint32_t ph = R.phi[b];
-        const float4 c = R.coords[b];
-        if (windowed && ((ph - lo) & 0xFFFFu) > width) break;
-        if (flagged(S, b)) continue;
-        if (!G::on(plane, c.x)) continue;
-        const float sc = scatter_of(c, xp, yp);
-        if (sc < cut && better(sc, b)) take(sc, b);
-    }
-}
+// No hit yet: above every (scatter, positions) key.
+constexpr unsigned long long kNoHit = ~0ull;
 
-template <class G, class Better, class Take, class HS>
-__device__ __forceinline__ void scan_window(const Smem& S, const Region<HS>& R, int b0, int nb, float xp,
-                                            float yp, float cut, float sqrt_cut, int plane,
-                                            Better better, Take take)
+// A straight line (last hit c0, difference d0) extrapolated to module t: the
+// least (scatter, position) over the module's unflagged hits under the scatter
+// cut; returns scatter bits << 32 | hi << 16 | position, or kNoHit.  Only the
+// hits from the bucket that holds the window's lower edge up to its upper edge
+// are visited: the bucket table replaces a binary search (seven dependent
+// loads a window of a 112-hit module), and hits before the edge in its bucket
+// cannot pass the cut, so looking at them changes nothing.  The search is
+// bound by the instructions of its longest lane (windows hold 2 to 3 hits on
+// average, the longest of a warp about ten), so the loop tests one key, the
+// scatter and the end; what concerns the few hits under the best scatter so
+// far stands in the branch.
+template <class G, class HS>
+__device__ __forceinline__ unsigned long long best_hit(const DevConfig& C, const Smem& S, const Region<HS>& R,
+                                                       int t, float3 c0, float3 d0, float cut, float sqrt_cut,
+                                                       uint32_t hi)
 {
-    if (nb <= 0) return;
-    uint32_t lo, width;
-    const bool windowed = window_of(xp, yp, cut, sqrt_cut, lo, width);
-    const int lo_idx = windowed ? lower_bound16(R.phi + b0, nb, lo) : 0;
-    scan_from<G>(S, R, b0, nb, xp, yp, cut, windowed, lo_idx, lo, width, plane, better, take);
+    const int b0 = S.modoff[t], b1 = S.modoff[t + 1];
+    float best = cut;
+    int bb = INT_MAX;
+    if (b0 < b1) {
+        for (int plane = 0; plane < G::kPlanes; plane++) {
+            float xp, yp;
+            extrapolate(c0, d0, G::z(C, t, plane), xp, yp);
+            uint32_t lo, width;
+            int b = b0;
+            // keys compared as phi16 << 16 | low bits; without a window every hit is inside
+            if (window_of(xp, yp, cut, sqrt_cut, lo, width)) {
+                constexpr uint32_t kIn = (1u << (16 - kBucketBits)) - 1u;
+                b = R.bucket[bucket_of(t, lo)];
+                b = b < b1 ? b : b0;
+                width = ((width + (lo & kIn)) << 16) | 0xFFFFu;
+                lo = (lo & ~kIn) << 16;
+            } else {
+                width = ~0u;
+            }
+            const int end = b;
+            do {
+                uint32_t key;
+                const float4 c = R.coords.get(b, key);
+                if (key - lo > width) break;
+                const float sc = scatter_of(c, xp, yp);
+                if (sc <= best && sc < cut && (sc < best || b < bb) && G::on(plane, c.x) && !flagged(S, b)) {
+                    best = sc;
+                    bb = b;
+                }
+                b = b + 1 < b1 ? b + 1 : b0;
+            } while (b != end);
+        }
+    }
+    return bb == INT_MAX ? kNoHit
+                         : ((unsigned long long)__float_as_uint(best) << 32) |
+                               (unsigned long long)((hi << 16) | (uint32_t)bb);
 }
 
 // First index in keys[0, n) whose upper 16 bits are >= v.
@@ -634,154 +687,76 @@ __device__ __forceinline__ int lower_bound_hi16(const uint32_t* keys, int n, uin
     return lo;
 }
 
-constexpr int kSeedBatch = 1;
+// Lanes that share one middle hit in seeding: each takes one of its
+// candidates, so K = 4 (the default) needs one round of extrapolations.  One
+// lane per middle hit used 8 to 11 lanes of a warp (the unflagged hits of a
+// module) for four extrapolations and scans in a row, the longest chain of a
+// step.  With the bucket table, search alone: one event 393 -> 266 us (128
+// threads), 16000 uneven events 6.22 -> 5.40 ms, 6000 module-pair events
+// 1.66 -> 1.12 ms.
+constexpr int kSeedLanes = 4;
+constexpr int kSeedGroups = 32 / kSeedLanes;
 
-// Candidates a[0, na) of one middle hit, processed together: extrapolations
-// to each plane of module i, then the binary searches of their windows in
-// lockstep (independent loads in flight), then the window scans.  Keeps the
-// best (scatter, a, b).
+// Seeding for middle hit c on module s+1 (c < 0: none) by kSeedLanes lanes:
+// the unflagged hits of module s nearest to c in phi (all hits at the K-th
+// smallest distance included), each extrapolated through c to module s+2,
+// where the unflagged hit of least scatter under the cut is sought; the kept
+// triplet minimises (scatter, position of a, position of b).  `outer` lists
+// the unflagged hits of module s in sorted order as (phi16 << 16 | position),
+// `nu` of them, so the nearest-first walk visits no flagged hit; the lanes
+// walk together and take the candidates in turn.  Every lane of the group
+// returns the triplet as scatter bits << 32 | a << 16 | b, or kNoHit.
 template <class G, class HS>
-__device__ __forceinline__ void seed_candidates(const DevConfig& C, const Smem& S, const Region<HS>& R,
-                                                int i, int i0, int ni, float4 Cc, float sqrt_cut,
-                                                const int* a, int na, bool& have, float& best_sc,
-                                                int& best_a, int& best_b)
+__device__ __forceinline__ unsigned long long seed_group(const DevConfig& C, const Smem& S,
+                                                         const Region<HS>& R, int s, int c,
+                                                         const uint32_t* outer, int nu, float sqrt_cut)
 {
-    for (int plane = 0; plane < G::kPlanes; plane++) {
-        const float zi = G::z(C, i, plane);
-        float xp[kSeedBatch], yp[kSeedBatch];
-        uint32_t lo[kSeedBatch], width[kSeedBatch];
-        int L[kSeedBatch], H[kSeedBatch];
-        bool win[kSeedBatch];
-#pragma unroll
-        for (int u = 0; u < kSeedBatch; u++) {
-            L[u] = 0;
-            H[u] = 0;
-            win[u] = false;
-            if (u < na) {
-                extrapolate(R.coords[a[u]], Cc, zi, xp[u], yp[u]);
-                win[u] = window_of(xp[u], yp[u], C.S_seed, sqrt_cut, lo[u], width[u]);
-                H[u] = win[u] ? ni : 0;
-            }
-        }
-        const uint16_t* phi = R.phi + i0;
-        for (int it = 0; it < 17; it++) {
-            bool active = false;
-#pragma unroll
-            for (int u = 0; u < kSeedBatch; u++) active |= L[u] < H[u];
-            if (!active) break;
-#pragma unroll
-            for (int u = 0; u < kSeedBatch; u++) {
-                if (L[u] < H[u]) {
-                    const int mid = (L[u] + H[u]) >> 1;
-                    if ((uint32_t)phi[mid] < lo[u])
-                        L[u] = mid + 1;
-                    else
-                        H[u] = mid;
+    unsigned long long best = kNoHit;
+    if (c >= 0) {
+        const int q = threadIdx.x & (kSeedLanes - 1);
+        const uint32_t phc = R.coords.phi(c);
+        int up = lower_bound_hi16(outer, nu, phc);
+        int dn = up - 1;
+        if (up == nu) up = 0;
+        if (dn < 0) dn = nu - 1;
+        uint32_t ku = outer[up], kd = outer[dn];
+        int found = 0, dK = INT_MAX;
+        bool more = true;
+        while (more) {
+            int a = -1;
+            for (int r = 0; r < kSeedLanes; r++) {
+                const int du = phi_dist(ku >> 16, phc), dd = phi_dist(kd >> 16, phc);
+                const bool take_up = du < dd || (du == dd && up <= dn);
+                const int d = take_up ? du : dd;
+                more = found < C.K || d <= dK;
+                if (!more) break;
+                if (++found == C.K) dK = d;
+                if (r == q) a = (int)((take_up ? ku : kd) & 0xFFFFu);
+                more = up != dn;  // else that was the last unflagged hit of the module
+                if (!more) break;
+                if (take_up) {
+                    up = up + 1 < nu ? up + 1 : 0;
+                    ku = outer[up];
+                } else {
+                    dn = dn > 0 ? dn - 1 : nu - 1;
+                    kd = outer[dn];
                 }
             }
+            if (a >= 0) {
+                const float4 Cc = R.coords[c];
+                const unsigned long long v = best_hit<G>(C, S, R, s + 2, make_float3(Cc.x, Cc.y, Cc.z),
+                                                         sub_rn(Cc, R.coords[a]), C.S_seed, sqrt_cut, (uint32_t)a);
+                best = v < best ? v : best;
+            }
         }
+    }
+    __syncwarp();
 #pragma unroll
-        for (int u = 0; u < kSeedBatch; u++) {
-            if (u >= na) continue;
-            const int au = a[u];
-            scan_from<G>(
-                S, R, i0, ni, xp[u], yp[u], C.S_seed, win[u], win[u] ? L[u] : 0, lo[u], width[u], plane,
-                [&](float sc, int b) {
-                    return !have || sc < best_sc ||
-                           (sc == best_sc && (au < best_a || (au == best_a && b < best_b)));
-                },
-                [&](float sc, int b) {
-                    have = true;
-                    best_sc = sc;
-                    best_a = au;
-                    best_b = b;
-                });
-        }
+    for (int o = 1; o < kSeedLanes; o <<= 1) {
+        const unsigned long long v = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+        best = v < best ? v : best;
     }
-}
-
-// Seeding for middle hit c on module s+1: the unflagged hits of module s
-// nearest to c in phi (all hits at the K-th smallest distance included),
-// each extrapolated through c to module s+2, where the unflagged hit of
-// least scatter under the cut is sought; the kept triplet minimises
-// (scatter, position of a, position of b).  `outer` lists the unflagged hits
-// of module s in sorted order as (phi16 << 16 | position), `nu` of them, so
-// the nearest-first walk visits no flagged hit.
-template <class G, class HS>
-__device__ bool seed_for(const DevConfig& C, const Smem& S, const Region<HS>& R, int s, int c,
-                         const uint32_t* outer, int nu, float sqrt_cut, int& oa, int& ob)
-{
-    const int i0 = S.modoff[s + 2], ni = S.modoff[s + 3] - i0;
-    if (nu <= 0 || ni <= 0) return false;
-    const uint32_t phc = R.phi[c];
-    const float4 Cc = R.coords[c];
-    const int j = lower_bound_hi16(outer, nu, phc);
-    int up = j, dn = j - 1;
-    int found = 0, dK = INT_MAX;
-    bool have = false;
-    float best_sc = 0.0f;
-    int best_a = 0, best_b = 0;
-    int cand[kSeedBatch];
-    int nc = 0;
-    for (int visited = 0; visited < nu; visited++) {
-        const int iu = up >= nu ? up - nu : up;
-        const int id = dn < 0 ? dn + nu : dn;
-        const uint32_t ku = outer[iu], kd = outer[id];
-        const int du = phi_dist(ku >> 16, phc);
-        const int dd = phi_dist(kd >> 16, phc);
-        int a, d;
-        if (du < dd || (du == dd && iu <= id)) {
-            a = (int)(ku & 0xFFFFu);
-            d = du;
-            up++;
-        } else {
-            a = (int)(kd & 0xFFFFu);
-            d = dd;
-            dn--;
-        }
-        if (found >= C.K && d > dK) break;
-        found++;
-        if (found == C.K) dK = d;
-        cand[nc++] = a;
-        if (nc == kSeedBatch) {
-            seed_candidates<G>(C, S, R, s + 2, i0, ni, Cc, sqrt_cut, cand, nc, have, best_sc, best_a, best_b);
-            nc = 0;
-        }
-    }
-    if (nc > 0)
-        seed_candidates<G>(C, S, R, s + 2, i0, ni, Cc, sqrt_cut, cand, nc, have, best_sc, best_a, best_b);
-    if (have) {
-        oa = best_a;
-        ob = best_b;
-    }
-    return have;
-}
-
-// Following: best unflagged hit on module t for the track's last two hits.
-template <class G, class HS>
-__device__ bool follow_best(const DevConfig& C, const Smem& S, const Region<HS>& R, int t, int h1, int h2,
-                            float sqrt_cut, int& cand, float& csc)
-{
-    const int b0 = S.modoff[t], nb = S.modoff[t + 1] - b0;
-    const float4 A = R.coords[h1], Cc = R.coords[h2];
-    bool have = false;
-    float best = 0.0f;
-    int bb = 0;
-    for (int plane = 0; plane < G::kPlanes; plane++) {
-        float xp, yp;
-        extrapolate(A, Cc, G::z(C, t, plane), xp, yp);
-        scan_window<G>(
-            S, R, b0, nb, xp, yp, C.S_follow, sqrt_cut, plane,
-            [&](float sc, int b) { return !have || sc < best || (sc == best && b < bb); },
-            [&](float sc, int b) {
-                have = true;
-                best = sc;
-                bb = b;
-            });
-    }
-    cand = bb;
-    csc = best;
-    return have;
+    return best;
 }
 
 __device__ __forceinline__ unsigned long long claim_key(unsigned long long tag, float score, int key)
@@ -834,12 +809,14 @@ __device__ __forceinline__ void follow_and_claim(const DevConfig& C, const Smem&
         T.cand = kDead;
         return;
     }
-    int b;
-    float sc;
-    if (follow_best<G>(C, S, R, t, T.h1, T.h2, sqrt_cut, b, sc)) {
+    const float4 L = R.coords[T.h2];
+    const unsigned long long best = best_hit<G>(C, S, R, t, make_float3(L.x, L.y, L.z), sub_rn(L, R.coords[T.h1]),
+                                                C.S_follow, sqrt_cut, 0u);
+    if (best != kNoHit) {
+        const int b = (int)(best & 0xFFFFu);
         T.cand = (uint16_t)b;
-        T.sc = sc;
-        const unsigned long long k = claim_key(tag, sc, T.key);
+        T.sc = __uint_as_float((uint32_t)(best >> 32));
+        const unsigned long long k = claim_key(tag, T.sc, T.key);
         atomicMin(&R.claim[b & R.cmask], k);
         if (T.nh == 3) {
             atomicMin(&R.claim[T.h0 & R.cmask], k);
@@ -855,10 +832,10 @@ __device__ __forceinline__ void follow_and_claim(const DevConfig& C, const Smem&
 // Iterative seeding and following.  Returns false (uniformly) on overflow.
 // Per module triplet (s, s+1, s+2) three phases separated by barriers:
 //   P0  work lists: unflagged middle hits of s+1, unflagged hits of s in order;
-//   P1  seeding and following of the forming tracks to t = s+3 with claims
-//       (every new seed searches its own continuation at once); threads take
-//       work items from a shared counter, seeds (the costlier items) first,
-//       so the step's barrier waits on a balanced tail;
+//   P1  seeding, kSeedLanes lanes per middle hit, and following of the forming
+//       tracks to t = s+3 with claims: a warp keeps its new seeds in its lanes
+//       and fills the other lanes with old tracks from a shared counter, so
+//       its following rounds are dense;
 //   P2  resolution of the claims, flags, termination.
 // Claims carry a tag (64 - t) << 48 above (scatter bits, track key), so a
 // claim of an earlier step always compares larger than one of the current
@@ -872,16 +849,6 @@ __device__ bool search_stage(const DevConfig& C, const Region<HS>& R, const Smem
     const int cap = C.fcap > 0 ? min(C.fcap, forming_capacity(n)) : forming_capacity(n);
     const float sq_seed = sqrtf(C.S_seed), sq_follow = sqrtf(C.S_follow);
     uint32_t* list = R.list;
-    if (tid == 0) {
-        misc[kCnt0] = 0;
-        misc[kCnt1] = 0;
-        misc[kNFin] = 0;
-        misc[kNTl] = 0;
-        misc[kErr] = 0;
-        misc[kList] = 0;
-        misc[kNew] = 0;
-    }
-    __syncthreads();
     int cur = 0;
     for (int s = 0; s + 2 <= M - 1; ++s) {
         const int nxt = cur ^ 1;
@@ -893,8 +860,6 @@ __device__ bool search_stage(const DevConfig& C, const Region<HS>& R, const Smem
             misc[kNew] = 0;
             misc[kWork] = 0;
         }
-        if (s + 3 <= M - 1)  // claim words of the target module start empty
-            for (int p = S.modoff[s + 3] + tid; p < S.modoff[s + 4]; p += NT) R.claim[p & R.cmask] = ~0ull;
         const int c0 = S.modoff[s + 1], c1 = S.modoff[s + 2];
         uint32_t* outer = list + (c1 - c0);
         for (int base = c0 + (tid & ~31); base < c1; base += NT) {
@@ -914,43 +879,64 @@ __device__ bool search_stage(const DevConfig& C, const Region<HS>& R, const Smem
                 const bool ok = a < o1 && !flagged(S, a);
                 const unsigned m = __ballot_sync(0xFFFFFFFFu, ok);
                 if (ok)
-                    outer[nu + __popc(m & ((1u << lane) - 1u))] =
-                        ((uint32_t)R.phi[a] << 16) | (uint32_t)a;
+                    outer[nu + __popc(m & ((1u << lane) - 1u))] = (R.coords.phi(a) << 16) | (uint32_t)a;
                 nu += __popc(m);
             }
             if (lane == 0) misc[kNOuter] = nu;
         }
         __syncthreads();
-        const int nl = misc[kList];
         const int nu = misc[kNOuter];
+        const int nl = nu > 0 && c1 < S.modoff[s + 3] ? misc[kList] : 0;
         const int nold = misc[kCnt0 + cur];
         const int t = s + 3;
         const bool follow = t <= M - 1;
         const unsigned long long tag = (unsigned long long)(64 - t) << 48;
         // P1
+        int na = 0, nc = -1, nb = 0;  // this lane's new seed
+        int i0 = (tid >> 5) * kSeedGroups, batch = 0;
         for (;;) {
-            const int i = atomicAdd(&misc[kWork], 1);
-            if (i >= nold + nl) break;
-            if (i >= nl) {
-                if (follow) {
-                    FTrack T = Fc[i - nl];
-                    follow_and_claim<G>(C, S, R, t, tag, sq_follow, T);
-                    Fc[i - nl] = T;
+            const bool seeding = i0 < nl;
+            if (seeding) {
+                const int i = i0 + lane / kSeedLanes;
+                const int c = i < nl ? (int)list[i] : -1;
+                const unsigned long long best = seed_group<G>(C, S, R, s, c, outer, nu, sq_seed);
+                if (best != kNoHit && lane % kSeedLanes == batch) {
+                    na = (int)(best >> 16) & 0xFFFF;
+                    nc = c;
+                    nb = (int)best & 0xFFFF;
                 }
-            } else {
-                const int c = (int)list[i];
-                int a, b;
-                if (seed_for<G>(C, S, R, s, c, outer, nu, sq_seed, a, b)) {
-                    const int slot = nold + atomicAdd(&misc[kNew], 1);
-                    if (slot < cap) {
-                        FTrack T = make_track(a, c, b, c, 3, 0);
-                        if (follow) follow_and_claim<G>(C, S, R, t, tag, sq_follow, T);
-                        Fc[slot] = T;
-                    } else {
-                        misc[kErr] = SBT_ERR_CAPACITY;
-                    }
-                }
+                i0 += NT / 32 * kSeedGroups;
+                // every lane of a group can hold a seed
+                if (++batch < kSeedLanes && i0 < nl) continue;
+                batch = 0;
             }
+            // following: this warp's new seeds, and old tracks in the other lanes
+            const unsigned idle = __ballot_sync(0xFFFFFFFFu, nc < 0);
+            int base = nold;
+            if (follow && idle) {
+                if (lane == 0) base = atomicAdd(&misc[kWork], __popc(idle));
+                base = __shfl_sync(0xFFFFFFFFu, base, 0);
+            }
+            int slot = base + __popc(idle & ((1u << lane) - 1u));
+            FTrack T;
+            if (nc >= 0) {
+                slot = nold + atomicAdd(&misc[kNew], 1);
+                T = make_track(na, nc, nb, nc, 3, 0);
+                if (slot >= cap) {
+                    misc[kErr] = SBT_ERR_CAPACITY;
+                    slot = -1;
+                }
+            } else if (slot < nold) {
+                T = Fc[slot];
+            } else {
+                slot = -1;
+            }
+            if (slot >= 0) {
+                if (follow) follow_and_claim<G>(C, S, R, t, tag, sq_follow, T);
+                Fc[slot] = T;
+            }
+            nc = -1;
+            if (!seeding && base + __popc(idle) >= nold) break;
         }
         __syncthreads();
         if (misc[kErr]) return false;
@@ -965,14 +951,14 @@ __device__ bool search_stage(const DevConfig& C, const Region<HS>& R, const Smem
                 if (T.cand != kNone) {
                     const unsigned long long k = claim_key(tag, T.sc, T.key);
                     // all claim words loaded at once (one round trip)
-                    const unsigned long long c0 = __ldcg(&R.claim[T.cand & R.cmask]);
-                    unsigned long long c1 = k, c2 = k, c3 = k;
+                    const unsigned long long ca = __ldcg(&R.claim[T.cand & R.cmask]);
+                    unsigned long long k0 = k, k1 = k, k2 = k;
                     if (T.nh == 3) {
-                        c1 = __ldcg(&R.claim[T.h0 & R.cmask]);
-                        c2 = __ldcg(&R.claim[T.h1 & R.cmask]);
-                        c3 = __ldcg(&R.claim[T.h2 & R.cmask]);
+                        k0 = __ldcg(&R.claim[T.h0 & R.cmask]);
+                        k1 = __ldcg(&R.claim[T.h1 & R.cmask]);
+                        k2 = __ldcg(&R.claim[T.h2 & R.cmask]);
                     }
-                    won = c0 == k && c1 == k && c2 == k && c3 == k;
+                    won = ca == k && k0 == k && k1 == k && k2 == k;
                 }
                 if (won) {
                     set_flag(S, T.cand);
@@ -1024,9 +1010,9 @@ __device__ void tracklet_filter(const DevConfig& C, const Region<HS>& R, const S
     // array, the tracklets' words cleared first
     for (int k = tid; k < ntl; k += NT) {
         const unsigned long long v = R.tracklets[k];
-        R.claim[v & 0xFFFF] = ~0ull;
-        R.claim[(v >> 16) & 0xFFFF] = ~0ull;
-        R.claim[(v >> 32) & 0xFFFF] = ~0ull;
+        R.claim_all[v & 0xFFFF] = ~0ull;
+        R.claim_all[(v >> 16) & 0xFFFF] = ~0ull;
+        R.claim_all[(v >> 32) & 0xFFFF] = ~0ull;
     }
     __syncthreads();
     for (int k = tid; k < ntl; k += NT) {
@@ -1046,9 +1032,9 @@ __device__ void tracklet_filter(const DevConfig& C, const Region<HS>& R, const S
             if (chi2 < C.C3) {
                 q = __float_as_uint(chi2);
                 unsigned long long kk = claim_key(0ull, chi2, key);
-                atomicMin(&R.claim[h[0]], kk);
-                atomicMin(&R.claim[h[1]], kk);
-                atomicMin(&R.claim[h[2]], kk);
+                atomicMin(&R.claim_all[h[0]], kk);
+                atomicMin(&R.claim_all[h[1]], kk);
+                atomicMin(&R.claim_all[h[2]], kk);
             }
         }
         R.tl_q[k] = q;
@@ -1060,7 +1046,7 @@ __device__ void tracklet_filter(const DevConfig& C, const Region<HS>& R, const S
         unsigned long long v = R.tracklets[k];
         int h0 = (int)(v & 0xFFFF), h1 = (int)((v >> 16) & 0xFFFF), h2 = (int)((v >> 32) & 0xFFFF);
         unsigned long long kk = claim_key(0ull, __uint_as_float(q), (int)(v >> 48));
-        if (__ldcg(&R.claim[h0]) == kk && __ldcg(&R.claim[h1]) == kk && __ldcg(&R.claim[h2]) == kk) {
+        if (__ldcg(&R.claim_all[h0]) == kk && __ldcg(&R.claim_all[h1]) == kk && __ldcg(&R.claim_all[h2]) == kk) {
             R.prev[h0] = kNone;
             R.prev[h1] = (uint16_t)h0;
             R.prev[h2] = (uint16_t)h1;
@@ -1096,7 +1082,7 @@ __device__ void output_stage(int e, int off, const Region<HS>& R, const Smem& S,
         for (int j = nh - 1; j >= 0; j--) {
             const int nq = R.prev[q];
             const float4 c = R.coords[q];
-            const int i = __float_as_int(c.w);
+            const int i = index_of(c);
             hits[u + j] = make_float4(c.x, c.y, c.z, __int_as_float(off + i));
             mn = i < mn ? i : mn;
             q = nq;
@@ -1135,7 +1121,7 @@ __device__ void run_event(const DevConfig& C, const Inputs& in, const Sorted& O,
         fail_event(e, st != SBT_OK ? st : SBT_ERR_CAPACITY, G, out);
         return;
     }
-    Region<HS> R = region_of<HS>(O, off, W, hb, r, cap);
+    Region<HS> R = region_of<HS>(O, C.M, e, off, W, hb, r, cap);
     for (int m = tid; m <= C.M; m += NT) S.modoff[m] = O.modoff[(int64_t)e * (C.M + 1) + m];
     for (int w = tid; w < (n + 31) / 32; w += NT) S.flag[w] = 0u;
     __syncthreads();
@@ -1144,18 +1130,20 @@ __device__ void run_event(const DevConfig& C, const Inputs& in, const Sorted& O,
     // them in a ring of the smallest power of two that covers every such span:
     // live positions never share a slot, and the ring stays in cache.  Without
     // such a power of two within the region's capacity, no ring.
-    if (tid == 0) {
+    if (tid < 32) {
         int w = 0;
-        for (int s = 0; s + 2 <= C.M - 1; s++)
+        for (int s = tid; s + 2 <= C.M - 1; s += 32)
             w = max(w, S.modoff[min(s + 4, C.M)] - S.modoff[max(s - 1, 0)]);
-        int p2 = 1;
-        while (p2 < w && p2 <= cap) p2 <<= 1;
-        S.misc[kCMask] = p2 >= w && p2 <= cap ? p2 - 1 : -1;
+        w = __reduce_max_sync(0xFFFFFFFFu, w);
+        const int p2 = w > 1 ? 1 << (32 - __clz(w - 1)) : 1;
+        if (tid == 0) S.misc[kCMask] = p2 <= cap ? p2 - 1 : -1;
+        if (tid < kMiscN && tid != kCMask && tid != kEvent) S.misc[tid] = 0;
     }
     __syncthreads();
+    // the ring starts empty; older claims lose against newer ones by their tag
     R.cmask = (unsigned)S.misc[kCMask];
-    // claim words of the modules that are never a following target
-    for (int p = tid; p < S.modoff[min(3, C.M)]; p += NT) R.claim[p & R.cmask] = ~0ull;
+    const int ring = R.cmask == ~0u ? n : min(n, (int)R.cmask + 1);
+    for (int p = tid; p < ring; p += NT) R.claim[p] = ~0ull;
     __syncthreads();
     if (!search_stage<NT, GEO>(C, R, S, n)) {
         fail_event(e, SBT_ERR_CAPACITY, G, out);
@@ -1485,8 +1473,9 @@ __global__ void k_debug_sort_copy(DevConfig C, Inputs in, Sorted O, uint16_t* ph
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < in.n_hits) {
-        phi16[i] = O.phi[i];
-        perm[i] = __float_as_int(HS::load((const typename HS::T*)O.coords, i).w);
+        const float4 c = HS::load((const typename HS::T*)O.coords, i);
+        phi16[i] = (uint16_t)(HS::key(c, O.phi, i) >> 16);
+        perm[i] = index_of(c);
     }
     if (i < (int64_t)in.n_events * (C.M + 1)) modoff[i] = O.modoff[i];
 }

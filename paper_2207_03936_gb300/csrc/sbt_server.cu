@@ -193,10 +193,11 @@ struct Slot {
 // Device bytes one batch needs (inputs, outputs and the plain workspace):
 // per hit 16 B inputs, 18 B sorted hits, about 45 B search scratch (claims,
 // links, lists, tracklets, forming and final tracks), about 12 B staging and
-// about 13 B outputs, rounded up.
+// about 13 B outputs, rounded up; per event its module offsets, counts and
+// bucket table.
 int64_t batch_bytes(int64_t hits, int64_t events)
 {
-    return hits * 112 + events * 320 + (1 << 16);
+    return hits * 112 + events * (320 + 2 * (sbt::kMaxModules << sbt::kBucketBits)) + (1 << 16);
 }
 
 }  // namespace

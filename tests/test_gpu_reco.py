@@ -601,6 +601,38 @@ def test_crowded_tiny_events_bit_exact(sbt, cfg_seed):
         h.close()
 
 
+@pytest.mark.parametrize("per_module", [1, 2, 31, 33, 100])
+@pytest.mark.parametrize("k", [1, 4, 5, 9])
+def test_candidate_lanes_and_bucket_windows_bit_exact(sbt, k, per_module):
+    """Seeding's lanes (K below, at and above the four lanes of a middle hit;
+    fewer outer hits than K; more middle hits than a warp's eight groups) and
+    the window scans from the bucket table (hits around phi = +-pi, where a
+    window runs from the last bucket to the first; several hits in one bucket;
+    a hit beside the axis, whose predictions get no window), on modules of
+    hits without tracks and wide cuts, so that most middle hits find triplets."""
+    rng = np.random.default_rng([k, per_module])
+    M, E = 7, 24
+    n = E * M * per_module
+    ang = np.where(rng.random(n) < 0.7, np.pi + rng.normal(0.0, 0.15, n), rng.uniform(0.0, 2 * np.pi, n))
+    r = np.where(rng.random(n) < 0.03, rng.uniform(0.0, 0.4, n), rng.uniform(5.1, 9.0, n))
+    module = np.tile(np.repeat(np.arange(M), per_module), E).astype(np.int32)
+    off = (np.arange(E + 1) * M * per_module).astype(np.int32)
+    perm = np.concatenate([off[e] + rng.permutation(M * per_module) for e in range(E)])
+    ev = synth.Events((r * np.cos(ang)).astype(np.float32), (r * np.sin(ang)).astype(np.float32),
+                      MZ[module], module[perm], off, np.full(n, -1, np.int32), 0, MZ[:M].copy())
+    ev.z = MZ[ev.module]
+    # the full modules' cut keeps an event's forming tracks under n / 12 + 64
+    cut = 0.3 if per_module < 64 else 0.02
+    cfg = dict(CFG, k_doublets=k, max_scatter_seed=cut, max_scatter_follow=0.2, max_chi2_tracklet=5000.0)
+    ref = oracle.reconstruct(ev.x, ev.y, ev.z, ev.module, ev.event_offsets, ev.module_z, oracle.config(**cfg))
+    h = sbt.sbt_create(ev.module_z, sbt.default_config(**cfg))
+    try:
+        for batched in (False, True):
+            assert_same(run_gpu(sbt, h, ev, batched), ref)
+    finally:
+        h.close()
+
+
 def test_event_ranges_outside_the_hits_are_reported(sbt, handle):
     # events whose hit range ends past n_hits get SBT_ERR_ARG on the device
     # and no tracks; the others are reconstructed as usual.  The hit arrays
