@@ -8,32 +8,68 @@
 // partial derivative at fixed line parameters (the parameters are stationary),
 //     d chi2 / d h' = 2 / sigma^2 (rx, ry, -(rx tx + ry ty)) = g,
 // chained through d h' / d(align_m): g itself for the translations, and
-// g . (dR_m/da v) for a rotation angle a, v = h - c_m.  Summed over the hits
-// of module m that is sum_ij (dR_m/da)_ij sum_h g_i v_j, so the kernel
-// accumulates per module g and the outer product g v^T (9 products a hit)
-// and the derivative matrices are applied once per module at the end.
+// g . (w x q) = w . (q x g) for a rotation angle, q = R_m (h - c_m) and w the
+// axis that the angle turns about: e_z for g, Rz e_y for b, Rz Ry e_x for a
+// (dR_m/d angle = [w]x R_m).  So the kernel accumulates per module the force g
+// and the torque q x g, and the axes are applied once per module at the end.
 //
-// Layout: one warp per track, lanes over its hits in rounds of 32.  A track
-// may have any number of hits and several hits on one module; a track
-// without a straight-line fit (fewer than two hits or modules) or with an
-// index out of range contributes nothing and is counted as skipped.  Each
-// warp owns an fp64 accumulator in shared memory, updated in a fixed lane
-// order; warps are summed in a fixed order per block and blocks in a fixed
-// order by the final kernel, so the result is bitwise reproducible.
-// Arithmetic is fp64 (the hits are fp32).
+// Arithmetic is fp64 (the hits are fp32), and the fp64 pipe is the bound: it
+// takes two lanes a clock and SM on this GPU, 16 clocks a warp instruction
+// whether its lanes are used or not, while 64 other warp instructions issue.
+// So every fp64 operation runs on full warps: a block takes tiles of
+// consecutive tracks and changes the assignment of threads between phases,
+//   hits    one thread per hit: aligned position p and q;
+//   tracks  one thread per track, tracks of a tile in order of length: the
+//           line, from the positions in shared memory;
+//   hits    one thread per hit: residuals, force and torque, stored in order of
+//           module (a stable counting sort of the tile's hits, integer work);
+//   modules one thread per (module, component): sums into a register that lives
+//           over all tiles.
+// 60 fp64 warp instructions per 32 hits; one warp per track with its lanes over
+// the hits took about 220 (20 of 32 lanes used, shuffled sums, five divisions
+// per track).  2.1 M tracks of 20 hits: 17.5 -> 5.2 ms, the fp64 pipe busy 76%
+// of the time; three hits a thread and tile (smaller tiles) 5.7 ms.
+//
+// A track may have any number of hits and several hits on one module (tracks
+// above kTileTrack hits go through a warp each); a track without a
+// straight-line fit (fewer than two hits or modules) or with an index out of
+// range contributes nothing and is counted as skipped.  Every sum has a fixed
+// order (hits of a module in tile order, tiles of a block, blocks), so the
+// result is bitwise reproducible.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "sbt_internal.h"
 
 namespace sbt {
 
-constexpr int kAdjThreads = 256;
+constexpr int kAdjThreads = 384;
 constexpr int kAdjWarps = kAdjThreads / 32;
-constexpr int kAdjBlocksPerSM = 4;
+constexpr int kAdjPerThread = 4;
+constexpr int kTileHits = kAdjThreads * kAdjPerThread;
+constexpr int kTileTracks = 128;  // 1536 hits are 77 tracks of average length
+constexpr int kTileTrack = 64;    // longest track of a tile (one hit per module at most, of 64)
+constexpr int kAdjPerModule = 6;  // force and torque
+constexpr int kAdjBlocksPerSM = 2;
+static_assert(kAdjPerModule * kMaxModules <= kAdjThreads, "one thread per accumulated component");
+static_assert(kTileTracks <= 256 && kMaxModules < 255 && kTileTrack <= kTileHits, "tile indices are bytes");
 
-int adjoint_blocks(int sm_count) { return kAdjBlocksPerSM * (sm_count > 0 ? sm_count : 1); }
+// Accumulated entries: per module force and torque, then chi2 and the
+// skipped-track count.
+__host__ __device__ inline int adjoint_entries(int M) { return kAdjPerModule * M + 2; }
+
+// Words per module of the angles' axes, after the blocks' entries.
+constexpr int kAdjAxes = 5;
+
+// Blocks of a launch: two per SM, fewer when there are fewer than 32 tracks
+// for each (a block's start, the rotation matrices, costs as much as 100
+// tracks).
+int adjoint_blocks(int sm_count, int n_tracks)
+{
+    return std::max(1, std::min(kAdjBlocksPerSM * std::max(sm_count, 1), (n_tracks + 31) / 32));
+}
 
 __device__ __forceinline__ double warp_sum(double v)
 {
@@ -42,273 +78,487 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-__device__ __forceinline__ void matvec(const double* R, double x, double y, double z, double& ox,
-                                       double& oy, double& oz)
+// Rotation of a module: R = Rz(g) Ry(b) Rx(a) in R[0..8], then the translation
+// with the plane's z added to its last component, sin g and cos g.
+constexpr int kAdjMat = 14;
+
+__device__ __forceinline__ void rotation(const double* th, double zc, double* R)
 {
-    ox = R[0] * x + R[1] * y + R[2] * z;
-    oy = R[3] * x + R[4] * y + R[5] * z;
-    oz = R[6] * x + R[7] * y + R[8] * z;
+    double sa, ca, sb, cb, sg, cg;
+    sincos(th[3], &sa, &ca);
+    sincos(th[4], &sb, &cb);
+    sincos(th[5], &sg, &cg);
+    R[0] = cg * cb;
+    R[1] = cg * sb * sa - sg * ca;
+    R[2] = cg * sb * ca + sg * sa;
+    R[3] = sg * cb;
+    R[4] = sg * sb * sa + cg * ca;
+    R[5] = sg * sb * ca - cg * sa;
+    R[6] = -sb;
+    R[7] = cb * sa;
+    R[8] = cb * ca;
+    R[9] = th[0];
+    R[10] = th[1];
+    R[11] = zc + th[2];
+    R[12] = sg;
+    R[13] = cg;
 }
 
-__device__ __forceinline__ void matmul(const double* A, const double* B, double* C)
-{
-    for (int i = 0; i < 3; i++)
-        for (int j = 0; j < 3; j++)
-            C[3 * i + j] = A[3 * i + 0] * B[0 + j] + A[3 * i + 1] * B[3 + j] + A[3 * i + 2] * B[6 + j];
-}
-
-// Per module: R = Rz Ry Rx and its derivatives with respect to a, b, g.
-__device__ void module_matrices(const double* th, double* out /* 36 */)
-{
-    double ca = cos(th[3]), sa = sin(th[3]);
-    double cb = cos(th[4]), sb = sin(th[4]);
-    double cg = cos(th[5]), sg = sin(th[5]);
-    double Rx[9] = {1, 0, 0, 0, ca, -sa, 0, sa, ca};
-    double dRx[9] = {0, 0, 0, 0, -sa, -ca, 0, ca, -sa};
-    double Ry[9] = {cb, 0, sb, 0, 1, 0, -sb, 0, cb};
-    double dRy[9] = {-sb, 0, cb, 0, 0, 0, -cb, 0, -sb};
-    double Rz[9] = {cg, -sg, 0, sg, cg, 0, 0, 0, 1};
-    double dRz[9] = {-sg, -cg, 0, cg, -sg, 0, 0, 0, 0};
-    double t1[9], t2[9];
-    matmul(Ry, Rx, t1);
-    matmul(Rz, t1, out + 0);        // R
-    matmul(Ry, dRx, t1);
-    matmul(Rz, t1, out + 9);        // dR/da
-    matmul(dRy, Rx, t1);
-    matmul(Rz, t1, out + 18);       // dR/db
-    matmul(Ry, Rx, t1);
-    matmul(dRz, t1, out + 27);      // dR/dg
-    (void)t2;
-}
-
-// One aligned hit: its module, the local coordinates v = h - c_m and the
-// aligned position p = R_m v + c_m + t_m.
+// Aligned hit: q = R (h - c), p = q + c + t.
 struct AHit {
-    double px, py, pz, vx, vy, vz;
-    int m;
+    double px, py, pz, qx, qy, qz;
 };
 
-__device__ __forceinline__ AHit aligned_hit(const DevConfig& C, const Inputs& in, const double* mats,
-                                            const double* align, int h)
+__device__ __forceinline__ AHit aligned_hit(const double* A, double zc, float x, float y, float z)
 {
+    const double vx = (double)x, vy = (double)y, vz = (double)z - zc;
     AHit a;
-    a.m = in.module[h];
-    const double* R = mats + 36 * a.m;
-    const double* th = align + 6 * a.m;
-    const double zc = (double)C.module_z[a.m];
-    a.vx = (double)in.x[h];
-    a.vy = (double)in.y[h];
-    a.vz = (double)in.z[h] - zc;
-    double ox, oy, oz;
-    matvec(R, a.vx, a.vy, a.vz, ox, oy, oz);
-    a.px = ox + th[0];
-    a.py = oy + th[1];
-    a.pz = oz + zc + th[2];
+    a.qx = A[0] * vx + A[1] * vy + A[2] * vz;
+    a.qy = A[3] * vx + A[4] * vy + A[5] * vz;
+    a.qz = A[6] * vx + A[7] * vy + A[8] * vz;
+    a.px = a.qx + A[9];
+    a.py = a.qy + A[10];
+    a.pz = a.qz + A[11];
     return a;
 }
 
-// Per-block accumulator entries: per module g (3) and g v^T (9), then chi2
-// and the skipped-track count.
-constexpr int kAdjPerModule = 12;
+struct Line {
+    double xm, ym, zm, tx, ty;
+};
 
-__host__ __device__ inline int adjoint_entries(int M) { return kAdjPerModule * M + 2; }
+// Residuals of an aligned hit, and its force and torque over 2 / sigma^2.
+__device__ __forceinline__ double force_torque(const AHit& a, const Line& l, double* f)
+{
+    const double dz = a.pz - l.zm;
+    const double rx = (a.px - l.xm) - l.tx * dz;
+    const double ry = (a.py - l.ym) - l.ty * dz;
+    const double w = rx * l.tx + ry * l.ty;
+    f[0] = rx;
+    f[1] = ry;
+    f[2] = -w;
+    f[3] = -(a.qy * w) - a.qz * ry;
+    f[4] = a.qz * rx + a.qx * w;
+    f[5] = a.qx * ry - a.qy * rx;
+    return rx * rx + ry * ry;
+}
 
-__global__ void __launch_bounds__(kAdjThreads) k_adjoint(DevConfig C, Inputs in,
-                                                          const int32_t* hit_offsets,
-                                                          const int32_t* track_hits,
-                                                          int32_t n_tracks, const double* align,
-                                                          double* partial, int want_grad)
+struct AdjSmem {
+    double tile[6 * kTileHits];   // p and q by hit (six arrays), then forces and torques by module order
+    double mats[kAdjMat * kMaxModules];
+    double zc[kMaxModules];
+    Line line[kTileTracks];
+    double warp_chi2[kAdjWarps];
+    int first[kTileTracks + 1];   // first tile hit of each track of the tile
+    int src[kTileTracks];         // first entry of track_hits of each track
+    int start[kMaxModules + 1];   // first hit of each module in module order
+    int skipped, n_tile, tile_end, has_long;
+    uint16_t before[kTileHits / 32 * kMaxModules];  // hits of a module in the earlier groups of 32
+    uint8_t count[kTileHits / 32 * kMaxModules];    // hits of a module in each group of 32
+    uint8_t module[kTileHits];    // by tile hit; 255: an index out of range
+    uint8_t order[kTileTracks];   // tracks by length
+    uint8_t skip[kTileTracks];
+    int bins[kTileTrack + 1];
+};
+static_assert(sizeof(double) * kAdjWarps * kAdjPerModule * kMaxModules <= sizeof(AdjSmem::tile),
+              "the long tracks' accumulators fit the tile");
+
+// One track above kTileTrack hits by one warp, lanes over its hits in rounds of
+// 32, positions recomputed in each pass; `my`: the warp's accumulators [6 M].
+__device__ void long_track(const Inputs& in, const AdjSmem& S, int M, const int32_t* hits, int n, double* my,
+                           double& chi2, int& skipped)
+{
+    const int lane = threadIdx.x & 31;
+    auto hit_at = [&](int j, int& m) {
+        const int h = hits[j];
+        m = in.module[h];
+        return aligned_hit(S.mats + kAdjMat * m, S.zc[m], in.x[h], in.y[h], in.z[h]);
+    };
+    bool bad = false;
+    int mlo = INT32_MAX, mhi = -1;
+    for (int j = lane; j < n; j += 32) {
+        const int h = hits[j];
+        const int m = h >= 0 && h < in.n_hits ? in.module[h] : -1;
+        bad |= m < 0 || m >= M;
+        mlo = min(mlo, m);
+        mhi = max(mhi, m);
+    }
+    bad = __any_sync(0xFFFFFFFFu, bad);
+    mlo = __reduce_min_sync(0xFFFFFFFFu, mlo);
+    mhi = __reduce_max_sync(0xFFFFFFFFu, mhi);
+    if (bad || mlo == mhi) {
+        if (lane == 0) skipped++;
+        return;
+    }
+    int m;
+    double sx = 0, sy = 0, sz = 0;
+    for (int j = lane; j < n; j += 32) {
+        const AHit a = hit_at(j, m);
+        sx += a.px;
+        sy += a.py;
+        sz += a.pz;
+    }
+    Line l;
+    l.xm = warp_sum(sx) / n;
+    l.ym = warp_sum(sy) / n;
+    l.zm = warp_sum(sz) / n;
+    double szz = 0, szx = 0, szy = 0;
+    for (int j = lane; j < n; j += 32) {
+        const AHit a = hit_at(j, m);
+        const double dz = a.pz - l.zm;
+        szz += dz * dz;
+        szx += dz * (a.px - l.xm);
+        szy += dz * (a.py - l.ym);
+    }
+    szz = warp_sum(szz);
+    l.tx = warp_sum(szx) / szz;
+    l.ty = warp_sum(szy) / szz;
+    for (int base = 0; base < n; base += 32) {
+        const int j = base + lane;
+        double f[kAdjPerModule];
+        m = -1 - lane;  // distinct for inactive lanes
+        if (j < n) chi2 += force_torque(hit_at(j, m), l, f);
+        // lanes that share a module add in lane order
+        const bool shared = __any_sync(0xFFFFFFFFu, __popc(__match_any_sync(0xFFFFFFFFu, m)) > 1);
+        for (int turn = 0; turn < (shared ? 32 : 1); turn++) {
+            if (j < n && (!shared || turn == lane))
+                for (int k = 0; k < kAdjPerModule; k++) my[kAdjPerModule * m + k] += f[k];
+            __syncwarp();
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kAdjThreads, kAdjBlocksPerSM)
+k_adjoint(DevConfig C, Inputs in, const int32_t* hit_offsets, const int32_t* track_hits, int32_t n_tracks,
+          const double* align, double* partial)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    AdjSmem& S = *(AdjSmem*)smem_raw;
     const int M = C.M;
-    const int P = adjoint_entries(M);
-    double* mats = (double*)smem_raw;               // [M][36]: R and its derivatives (R used here)
-    double* acc = mats + 36 * M;                    // [warps][P]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int m = tid; m < M; m += kAdjThreads) module_matrices(align + 6 * m, mats + 36 * m);
-    for (int k = tid; k < kAdjWarps * P; k += kAdjThreads) acc[k] = 0.0;
+    if (tid < M) {
+        double* A = S.mats + kAdjMat * tid;
+        S.zc[tid] = (double)C.module_z[tid];
+        rotation(align + 6 * tid, S.zc[tid], A);
+        if (blockIdx.x == 0) {  // the axes of the angles, for the reduction
+            double* x = partial + (int64_t)gridDim.x * adjoint_entries(M) + kAdjAxes * tid;
+            x[0] = A[0];  // Rz Ry e_x: the first column of R
+            x[1] = A[3];
+            x[2] = A[6];
+            x[3] = -A[12];  // Rz e_y = (-sin g, cos g, 0)
+            x[4] = A[13];
+        }
+    }
+    if (tid == 0) {
+        S.skipped = 0;
+        S.has_long = 0;
+    }
     __syncthreads();
-    double* my = acc + warp * P;
-    const double s2 = (double)C.sigma * (double)C.sigma;
-    const double inv_s2 = 1.0 / s2, two_inv_s2 = 2.0 * inv_s2;  // one fp64 division per launch
-    const int gw = blockIdx.x * kAdjWarps + warp;
-    const int nw = gridDim.x * kAdjWarps;
     const int64_t end = n_tracks > 0 ? hit_offsets[n_tracks] : 0;
-    for (int t = gw; t < n_tracks; t += nw) {
-        const int h0 = hit_offsets[t];
-        const int n = hit_offsets[t + 1] - h0;
-        // every lane reads the same offsets, so these branches are uniform
-        if (n < 2 || h0 < 0 || (int64_t)h0 + n > end) {
-            if (lane == 0) my[P - 1] += 1.0;
-            continue;
-        }
-        // pass 1: validity, sums; hits 0..63 kept in registers (two per lane)
-        AHit keep0, keep1;
-        bool bad = false;
-        int mlo = INT32_MAX, mhi = -1;
-        double sx = 0, sy = 0, sz = 0;
-        for (int base = 0; base < n; base += 32) {
-            const int j = base + lane;
-            if (j >= n) continue;
-            const int h = track_hits[h0 + j];
-            if (h < 0 || h >= in.n_hits || in.module[h] < 0 || in.module[h] >= M) {
-                bad = true;
-                continue;
+    const int tbeg = (int)((int64_t)n_tracks * blockIdx.x / gridDim.x);
+    const int tend = (int)((int64_t)n_tracks * (blockIdx.x + 1) / gridDim.x);
+    double acc = 0.0, chi2 = 0.0;  // this thread's (module, component), and its hits' squared residuals
+    int skipped = 0;
+    int t0 = tbeg;
+    while (t0 < tend) {
+        // the tile: the next tracks whose hits fit, at most kTileTracks of
+        // them (scan over four warps); skipped and long ones take no room
+        if (tid < kTileTracks) {
+            const int t = t0 + tid;
+            int n = 0, h0 = 0;
+            if (t < tend) {
+                h0 = hit_offsets[t];
+                n = hit_offsets[t + 1] - h0;
+                const bool bad = n < 2 || h0 < 0 || (int64_t)h0 + n > end;
+                if (!bad && n > kTileTrack) S.has_long = 1;
+                if (bad || n > kTileTrack) n = bad ? -1 : 0;
             }
-            const AHit a = aligned_hit(C, in, mats, align, h);
-            if (base == 0)
-                keep0 = a;
-            else if (base == 32)
-                keep1 = a;
-            mlo = min(mlo, a.m);
-            mhi = max(mhi, a.m);
-            sx += a.px;
-            sy += a.py;
-            sz += a.pz;
-        }
-        bad = __any_sync(0xFFFFFFFFu, bad);
+            S.skip[tid] = n < 0;
+            n = max(n, 0);
+            S.src[tid] = h0;
+            int incl = n;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            mlo = min(mlo, __shfl_xor_sync(0xFFFFFFFFu, mlo, o));
-            mhi = max(mhi, __shfl_xor_sync(0xFFFFFFFFu, mhi, o));
-        }
-        if (bad || mlo == mhi) {
-            if (lane == 0) my[P - 1] += 1.0;
-            continue;
-        }
-        auto hit_at = [&](int base, int j) -> AHit {
-            if (base == 0) return keep0;
-            if (base == 32) return keep1;
-            return aligned_hit(C, in, mats, align, track_hits[h0 + j]);
-        };
-        sx = warp_sum(sx);
-        sy = warp_sum(sy);
-        sz = warp_sum(sz);
-        const double xm = sx / n, ym = sy / n, zm = sz / n;
-        // pass 2: second moments
-        double szz = 0, szx = 0, szy = 0;
-        for (int base = 0; base < n; base += 32) {
-            const int j = base + lane;
-            if (j >= n) continue;
-            const AHit a = hit_at(base, j);
-            const double dz = a.pz - zm;
-            szz += dz * dz;
-            szx += dz * (a.px - xm);
-            szy += dz * (a.py - ym);
-        }
-        szz = warp_sum(szz);
-        szx = warp_sum(szx);
-        szy = warp_sum(szy);
-        const double tx = szx / szz, ty = szy / szz;
-        // pass 3: residuals, chi2 and the gradient per module; lanes of one
-        // round that share a module add in lane order
-        double c2 = 0;
-        for (int base = 0; base < n; base += 32) {
-            const int j = base + lane;
-            const bool act = j < n;
-            double g[kAdjPerModule];
-            int m = -1 - lane;  // distinct for inactive lanes
-            if (act) {
-                const AHit a = hit_at(base, j);
-                m = a.m;
-                const double dz = a.pz - zm;
-                const double rx = (a.px - xm) - tx * dz;
-                const double ry = (a.py - ym) - ty * dz;
-                c2 += (rx * rx + ry * ry) * inv_s2;
-                g[0] = rx * two_inv_s2;
-                g[1] = ry * two_inv_s2;
-                g[2] = -(rx * tx + ry * ty) * two_inv_s2;
-                const double v[3] = {a.vx, a.vy, a.vz};
-#pragma unroll
-                for (int i = 0; i < 3; i++)
-#pragma unroll
-                    for (int k = 0; k < 3; k++) g[3 + 3 * i + k] = g[i] * v[k];
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                if (lane >= o) incl += v;
             }
-            if (want_grad) {
-                const unsigned same = __match_any_sync(0xFFFFFFFFu, m);
-                if (!__any_sync(0xFFFFFFFFu, __popc(same) > 1)) {
-                    if (act) {
+            S.first[tid + 1] = incl;
+        }
+        if (tid <= kTileTrack) S.bins[tid] = 0;
+        __syncthreads();
+        int before = 0;
+        if (tid < kTileTracks)
+            for (int w = 0; w < warp; w++) before += S.first[32 * w + 32];
+        __syncthreads();
+        if (tid < kTileTracks) {
+            const int e = S.first[tid + 1] + before;
+            const int b = __shfl_up_sync(0xFFFFFFFFu, e, 1);
+            const int s = lane > 0 ? b : before;
+            // tracks that fit form a prefix
+            S.first[tid + 1] = e;
+            if (t0 + tid < tend && e <= kTileHits) {
+                atomicAdd(&S.bins[kTileTrack - (e - s)], 1);
+                if (S.skip[tid]) skipped++;
+            }
+            if (tid == 0) S.first[0] = 0;
+        }
+        __syncthreads();
+        if (tid < kTileTracks) {
+            const bool fits = t0 + tid < tend && S.first[tid + 1] <= kTileHits;
+            const bool next = tid + 1 < kTileTracks && t0 + tid + 1 < tend && S.first[min(tid + 2, kTileTracks)] <= kTileHits;
+            if (fits && !next) {
+                S.n_tile = tid + 1;
+                S.tile_end = S.first[tid + 1];
+            }
+        }
+        if (tid == 0)  // longest tracks first
+            for (int k = 0, s = 0; k <= kTileTrack; k++) {
+                const int c = S.bins[k];
+                S.bins[k] = s;
+                s += c;
+            }
+        for (int k = tid; k < kTileHits / 32 * M; k += kAdjThreads) S.count[k] = 0;
+        __syncthreads();
+        const int nt = S.n_tile, nh = S.tile_end;
+        if (tid < nt) S.order[atomicAdd(&S.bins[kTileTrack - (S.first[tid + 1] - S.first[tid])], 1)] = (uint8_t)tid;
+        // hits: track, module, aligned position, rank within the module's hits
+        // of this group of 32
+        uint32_t mine[kAdjPerThread];  // module | track << 8 | rank << 16; module 255: no hit
 #pragma unroll
-                        for (int k = 0; k < kAdjPerModule; k++) my[kAdjPerModule * m + k] += g[k];
-                    }
-                } else {
-                    for (int l = 0; l < 32; l++) {
-                        if (lane == l && act) {
-#pragma unroll
-                            for (int k = 0; k < kAdjPerModule; k++) my[kAdjPerModule * m + k] += g[k];
-                        }
-                        __syncwarp();
-                    }
+        for (int u = 0; u < kAdjPerThread; u++) {
+            const int h = tid + u * kAdjThreads;
+            int m = 255, tr = 0;
+            if (h < nh) {
+                int hi = nt;  // last track that starts at or before h and is not empty
+                while (hi - tr > 1) {
+                    const int mid = (tr + hi) >> 1;
+                    if (S.first[mid] <= h)
+                        tr = mid;
+                    else
+                        hi = mid;
                 }
-                __syncwarp();
+                const int i = track_hits[S.src[tr] + (h - S.first[tr])];
+                if (i >= 0 && i < in.n_hits) {
+                    const int mm = in.module[i];
+                    if (mm >= 0 && mm < M) m = mm;
+                }
+                S.module[h] = (uint8_t)m;
+                if (m != 255) {
+                    const AHit a = aligned_hit(S.mats + kAdjMat * m, S.zc[m], in.x[i], in.y[i], in.z[i]);
+                    S.tile[0 * kTileHits + h] = a.px;
+                    S.tile[1 * kTileHits + h] = a.py;
+                    S.tile[2 * kTileHits + h] = a.pz;
+                    S.tile[3 * kTileHits + h] = a.qx;
+                    S.tile[4 * kTileHits + h] = a.qy;
+                    S.tile[5 * kTileHits + h] = a.qz;
+                }
+            }
+            const unsigned same = __match_any_sync(0xFFFFFFFFu, m);
+            const int rank = __popc(same & ((1u << lane) - 1u));
+            if (m != 255 && rank == 0) S.count[(h >> 5) * M + m] = (uint8_t)__popc(same);
+            mine[u] = (uint32_t)m | ((uint32_t)tr << 8) | ((uint32_t)rank << 16);
+        }
+        __syncthreads();
+        // tracks: the line (tid < nt); modules: hits before each group (the
+        // last warps, integer work beside the fp64 of the first)
+        if (tid < nt) {
+            const int tr = S.order[tid];
+            const int b = S.first[tr], n = S.first[tr + 1] - b;
+            bool bad = false, one = true;
+            const double* P = S.tile + b;
+            // sums of four join the sums of all: means and slopes (times 200 mm
+            // of dz) carry the rounding that the residuals feel, and a plain
+            // sum left 20% more of it in the gradient than the shuffled one
+            double sx = 0, sy = 0, sz = 0;
+            for (int j = 0; j < n; j += 4) {
+                double x = 0, y = 0, z = 0;
+#pragma unroll
+                for (int u = 0; u < 4; u++)
+                    if (j + u < n) {
+                        bad |= S.module[b + j + u] == 255;
+                        one &= S.module[b + j + u] == S.module[b];
+                        x += P[0 * kTileHits + j + u];
+                        y += P[1 * kTileHits + j + u];
+                        z += P[2 * kTileHits + j + u];
+                    }
+                sx += x;
+                sy += y;
+                sz += z;
+            }
+            if (n > 0 && (bad || one)) {
+                S.skip[tr] = 1;
+                skipped++;
+            } else if (n > 0) {
+                Line l;
+                l.xm = sx / n;
+                l.ym = sy / n;
+                l.zm = sz / n;
+                double szz = 0, szx = 0, szy = 0;
+                for (int j = 0; j < n; j += 4) {
+                    double zz = 0, zx = 0, zy = 0;
+#pragma unroll
+                    for (int u = 0; u < 4; u++)
+                        if (j + u < n) {
+                            const double dz = P[2 * kTileHits + j + u] - l.zm;
+                            zz += dz * dz;
+                            zx += dz * (P[0 * kTileHits + j + u] - l.xm);
+                            zy += dz * (P[1 * kTileHits + j + u] - l.ym);
+                        }
+                    szz += zz;
+                    szx += zx;
+                    szy += zy;
+                }
+                l.tx = szx / szz;
+                l.ty = szy / szz;
+                S.line[tr] = l;
             }
         }
-        c2 = warp_sum(c2);
-        if (lane == 0) my[P - 2] += c2;
-        __syncwarp();
-    }
-    __syncthreads();
-    for (int k = tid; k < P; k += kAdjThreads) {
-        double s = 0;
-        for (int w = 0; w < kAdjWarps; w++) s += acc[w * P + k];
-        partial[(int64_t)blockIdx.x * P + k] = s;
-    }
-}
-
-// Fixed-order sum of the blocks' entries, then per module: the translation
-// gradient is the summed g, each rotation gradient sum_ij (dR/d angle)_ij
-// (sum g v^T)_ij.  One block of kAdjReduceThreads >= 12 M + 2 threads.
-constexpr int kAdjReduceThreads = 1024;
-static_assert(kAdjReduceThreads >= kAdjPerModule * kMaxModules + 2, "one thread per accumulator entry");
-
-__global__ void __launch_bounds__(kAdjReduceThreads) k_adjoint_reduce(int M, int blocks, const double* partial,
-                                                                      const double* align, double* chi2_sum,
-                                                                      double* grad, int32_t* skipped)
-{
-    __shared__ double s[kAdjPerModule * kMaxModules + 2];
-    const int P = adjoint_entries(M);
-    for (int k = threadIdx.x; k < P; k += blockDim.x) {
-        double v = 0;
-        for (int b = 0; b < blocks; b++) v += partial[(int64_t)b * P + k];
-        s[k] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < M && grad) {
-        const int m = threadIdx.x;
-        double D[36];
-        module_matrices(align + 6 * m, D);
-        const double* a = s + kAdjPerModule * m;
-        grad[6 * m + 0] = a[0];
-        grad[6 * m + 1] = a[1];
-        grad[6 * m + 2] = a[2];
-        for (int r = 0; r < 3; r++) {
-            const double* dR = D + 9 * (r + 1);
-            double v = 0;
-            for (int ij = 0; ij < 9; ij++) v += dR[ij] * a[3 + ij];
-            grad[6 * m + 3 + r] = v;
+        if (tid >= kAdjThreads - 64 && tid - (kAdjThreads - 64) < M) {
+            const int m = tid - (kAdjThreads - 64);
+            int s = 0;
+#pragma unroll 8
+            for (int g = 0; g < kTileHits / 32; g++) {
+                S.before[g * M + m] = (uint16_t)s;
+                s += S.count[g * M + m];
+            }
+            S.start[m + 1] = s;
         }
+        __syncthreads();
+        if (warp == 0) {  // module starts, two modules a lane
+            const int a = 2 * lane < M ? S.start[2 * lane + 1] : 0, b = 2 * lane + 1 < M ? S.start[2 * lane + 2] : 0;
+            int incl = a + b;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            if (2 * lane < M) S.start[2 * lane + 1] = incl - b;
+            if (2 * lane + 1 < M) S.start[2 * lane + 2] = incl;
+            if (lane == 0) S.start[0] = 0;
+        }
+        // hits: forces and torques, kept in registers until every position is
+        // read, then stored in module order over the positions
+        double f[kAdjPerThread][kAdjPerModule];
+#pragma unroll
+        for (int u = 0; u < kAdjPerThread; u++) {
+            const int h = tid + u * kAdjThreads;
+            const int tr = (int)(mine[u] >> 8) & 0xFF;
+#pragma unroll
+            for (int k = 0; k < kAdjPerModule; k++) f[u][k] = 0.0;
+            if ((mine[u] & 0xFFu) != 255u && !S.skip[tr]) {
+                AHit a;
+                a.px = S.tile[0 * kTileHits + h];
+                a.py = S.tile[1 * kTileHits + h];
+                a.pz = S.tile[2 * kTileHits + h];
+                a.qx = S.tile[3 * kTileHits + h];
+                a.qy = S.tile[4 * kTileHits + h];
+                a.qz = S.tile[5 * kTileHits + h];
+                chi2 += force_torque(a, S.line[tr], f[u]);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kAdjPerThread; u++) {
+            const int h = tid + u * kAdjThreads;
+            const int m = (int)(mine[u] & 0xFFu);
+            if (m != 255) {
+                const int s = S.start[m] + S.before[(h >> 5) * M + m] + (int)(mine[u] >> 16);
+#pragma unroll
+                for (int k = 0; k < kAdjPerModule; k++) S.tile[kAdjPerModule * s + k] = f[u][k];
+            }
+        }
+        __syncthreads();
+        if (tid < kAdjPerModule * M) {
+            const int m = tid / kAdjPerModule, k = tid % kAdjPerModule;
+            const int e = S.start[m + 1];
+            for (int s = S.start[m]; s < e; s++) acc += S.tile[kAdjPerModule * s + k];
+        }
+        t0 += nt;
+        __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        *chi2_sum = s[P - 2];
-        if (skipped) *skipped = (int32_t)s[P - 1];
+    if (S.has_long) {
+        for (int k = tid; k < kAdjWarps * kAdjPerModule * M; k += kAdjThreads) S.tile[k] = 0.0;
+        __syncthreads();
+        for (int t = tbeg + warp; t < tend; t += kAdjWarps) {
+            const int h0 = hit_offsets[t], n = hit_offsets[t + 1] - h0;
+            if (n > kTileTrack && h0 >= 0 && (int64_t)h0 + n <= end)
+                long_track(in, S, M, track_hits + h0, n, S.tile + warp * kAdjPerModule * M, chi2, skipped);
+        }
+        __syncthreads();
+        if (tid < kAdjPerModule * M)
+            for (int w = 0; w < kAdjWarps; w++) acc += S.tile[w * kAdjPerModule * M + tid];
+    }
+    // the block's entries
+    const int P = adjoint_entries(M);
+    if (skipped) atomicAdd(&S.skipped, skipped);
+    chi2 = warp_sum(chi2);
+    if (lane == 0) S.warp_chi2[warp] = chi2;
+    __syncthreads();
+    double* out = partial + (int64_t)blockIdx.x * P;
+    const double s2 = (double)C.sigma * (double)C.sigma;
+    if (tid < kAdjPerModule * M) out[tid] = acc * (2.0 / s2);
+    if (tid == 0) {
+        double c = 0.0;
+        for (int w = 0; w < kAdjWarps; w++) c += S.warp_chi2[w];
+        out[P - 2] = c / s2;
+        out[P - 1] = (double)S.skipped;
     }
 }
 
-size_t adjoint_partial_entries(int M, int blocks) { return (size_t)blocks * (size_t)adjoint_entries(M); }
+// Sum of the blocks' entries in a fixed order, one block per module (and one
+// for chi2 and the skipped count): 64 threads per entry over the blocks, then
+// a tree.  The translation gradient is the summed force, each rotation
+// gradient the torque along the angle's axis.
+constexpr int kAdjRows = 64;
+
+__global__ void __launch_bounds__(8 * kAdjRows)
+k_adjoint_reduce(int M, int blocks, const double* partial, double* chi2_sum, double* grad, int32_t* skipped)
+{
+    __shared__ double s[kAdjRows][8];
+    const int P = adjoint_entries(M);
+    const int m = blockIdx.x, k = threadIdx.x & 7, row = threadIdx.x >> 3;
+    const int n = m < M ? kAdjPerModule : 2;
+    double v = 0.0;
+    if (k < n)
+        for (int b = row; b < blocks; b += kAdjRows) v += partial[(int64_t)b * P + kAdjPerModule * m + k];
+    s[row][k] = v;
+    __syncthreads();
+    for (int o = kAdjRows / 2; o > 0; o >>= 1) {
+        if (row < o) s[row][k] += s[row + o][k];
+        __syncthreads();
+    }
+    if (threadIdx.x != 0) return;
+    const double* a = s[0];
+    if (m == M) {
+        *chi2_sum = a[0];
+        if (skipped) *skipped = (int32_t)a[1];
+    } else if (grad) {
+        double* g = grad + 6 * m;
+        g[0] = a[0];
+        g[1] = a[1];
+        g[2] = a[2];
+        const double* x = partial + (int64_t)blocks * P + kAdjAxes * m;
+        g[3] = x[0] * a[3] + x[1] * a[4] + x[2] * a[5];
+        g[4] = x[3] * a[3] + x[4] * a[4];
+        g[5] = a[5];  // e_z
+    }
+}
+
+size_t adjoint_partial_entries(int M, int blocks)
+{
+    return (size_t)blocks * (size_t)adjoint_entries(M) + (size_t)kAdjAxes * M;
+}
 
 cudaError_t launch_adjoint(const DevConfig& C, const Inputs& in, const int32_t* hit_offsets,
                            const int32_t* track_hits, int32_t n_tracks, const double* align,
                            double* chi2_sum, double* grad, int32_t* skipped, const AdjointWork& W,
                            cudaStream_t stream)
 {
-    const int M = C.M;
-    size_t sm = sizeof(double) * (36 * (size_t)M + (size_t)kAdjWarps * adjoint_entries(M));
     cudaError_t err = cudaFuncSetAttribute(k_adjoint, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)sm);
+                                           (int)sizeof(AdjSmem));
     if (err != cudaSuccess) return err;
-    k_adjoint<<<W.blocks, kAdjThreads, sm, stream>>>(C, in, hit_offsets, track_hits, n_tracks,
-                                                      align, W.partial, grad != nullptr);
-    k_adjoint_reduce<<<1, kAdjReduceThreads, 0, stream>>>(M, W.blocks, W.partial, align, chi2_sum, grad, skipped);
+    k_adjoint<<<W.blocks, kAdjThreads, sizeof(AdjSmem), stream>>>(C, in, hit_offsets, track_hits, n_tracks, align,
+                                                                   W.partial);
+    k_adjoint_reduce<<<C.M + 1, 8 * kAdjRows, 0, stream>>>(C.M, W.blocks, W.partial, chi2_sum, grad, skipped);
     return cudaGetLastError();
 }
 

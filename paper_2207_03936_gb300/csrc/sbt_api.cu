@@ -826,7 +826,7 @@ sbt_status sbt_fit_adjoint(sbt_handle* h, const float* x, const float* y, const 
     if (!hit_offsets || !align || !chi2_sum || (n_tracks > 0 && (!track_hits || !x || !y || !z || !module)))
         return fail(h, SBT_ERR_ARG, "NULL argument");
     AdjointWork W;
-    W.blocks = adjoint_blocks(h->sm_count);
+    W.blocks = adjoint_blocks(h->sm_count, n_tracks);
     size_t need = sizeof(double) * adjoint_partial_entries(h->C.M, W.blocks);
     cudaError_t e = h->misc_arena.reserve(std::max(need, h->misc_arena.bytes));
     if (e != cudaSuccess) return cuda_fail(h, e, "adjoint allocation");

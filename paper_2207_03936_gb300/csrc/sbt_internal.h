@@ -144,7 +144,7 @@ cudaError_t launch_adjoint(const DevConfig& C, const Inputs& in, const int32_t* 
                            const int32_t* track_hits, int32_t n_tracks, const double* align,
                            double* chi2_sum, double* grad, int32_t* skipped, const AdjointWork& W,
                            cudaStream_t stream);
-int adjoint_blocks(int sm_count);
+int adjoint_blocks(int sm_count, int n_tracks);
 size_t adjoint_partial_entries(int M, int blocks);
 
 // Handle accessors for translation units that cannot see the handle type.

@@ -126,3 +126,35 @@ def test_adjoint_on_long_repeated_and_invalid_tracks(setup):
     # reproducible to the bit with the repeated-module path taken
     c2, g2, _ = sbt.sbt_fit_adjoint(h, *d, torch.from_numpy(align).cuda(), with_skipped=True)
     assert torch.equal(c.cpu(), c2.cpu()) and np.array_equal(g, g2.cpu().numpy())
+
+
+@pytest.mark.parametrize("lengths", [[3], [2, 1, 0], [64], [65, 64, 2, 63], [20, 24, 17, 33], [200, 3, 5]],
+                         ids=lambda v: "-".join(map(str, v)))
+@pytest.mark.parametrize("n_tracks", [1, 31, 129, 2000])
+def test_adjoint_tiles(setup, n_tracks, lengths):
+    """Tiles of tracks by hits and by number (1536 hits, 128 tracks: full,
+    exceeded, one short), tracks at and above the longest of a tile, tracks
+    without a fit in between, fewer tracks than blocks; random hits, so that
+    modules repeat within tracks."""
+    sbt, h, ev, _, _, d = setup
+    rng = np.random.default_rng([n_tracks, *lengths])
+    n = np.resize(np.array(lengths), n_tracks)
+    ho = np.concatenate([[0], np.cumsum(n)]).astype(np.int32)
+    th = rng.integers(0, ev.n_hits, int(ho[-1])).astype(np.int32)
+    if n_tracks > 100 and len(th) > 500:
+        th[len(th) // 2] = ev.n_hits      # one track with an index out of range
+    align = np.concatenate([rng.normal(0, 0.005, (52, 3)), rng.normal(0, 5e-5, (52, 3))], 1)
+    args = [d["x"], d["y"], d["z"], d["m"], torch.from_numpy(ho).cuda(), torch.from_numpy(th).cuda(),
+            torch.from_numpy(align).cuda()]
+    c, g, sk = sbt.sbt_fit_adjoint(h, *args, with_skipped=True)
+    c2, g2 = sbt.sbt_fit_adjoint(h, *args)
+    v, go, so = oracle.align_chi2(ev.x, ev.y, ev.z, ev.module, ho, th, ev.module_z, align, SIGMA,
+                                  count_skipped=True)
+    assert int(sk.item()) == so
+    # residuals of centimetres: the fp64 sums agree to a few thousand roundings;
+    # residuals that vanish (two hits) are left with about ten roundings of
+    # coordinates up to 750 mm, delta = 1e-12 mm a hit, at lever arms up to 42 mm
+    delta, hits = 1e-12, len(th)
+    assert abs(float(c.item()) - v) <= 1e-12 * v + hits * (delta / SIGMA) ** 2
+    assert np.abs(g.cpu().numpy() - go).max() <= 1e-11 * np.abs(go).max() + hits * 2 * delta / SIGMA ** 2 * 42
+    assert torch.equal(c, c2) and torch.equal(g, g2)
