@@ -79,7 +79,7 @@ typedef struct {
     float hit_sigma;             /* hit resolution for chi2, mm; default 0.012 */
     int32_t max_hits_per_event;  /* events with more hits get SBT_ERR_CAPACITY; default and maximum 16384 */
     int32_t max_forming_tracks;  /* forming tracks alive per event: n_hits/12 + 64; a positive value lowers the bound */
-    int32_t threads_per_block;   /* 64, 128 or 256; 0 = 128 (batched: autotuned value if any) */
+    int32_t threads_per_block;   /* 64, 128 or 256; 0 = by the number of events (batched: autotuned value if any) */
     int32_t gec_max_hits;        /* global event cut (the paper's VELO sequence, first step): events
                                     with more hits are rejected unreconstructed (event status
                                     SBT_EVENT_CUT); 0 = no cut (default) */

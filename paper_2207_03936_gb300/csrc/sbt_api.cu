@@ -155,6 +155,7 @@ struct sbt_handle {
     int sm_count = 0;
     std::string err;
     Arena plain_arena, pers_arena, stage_arena, host_arena, misc_arena, sorted_arena;
+    int concurrent = 1;     // calls of other handles that share the GPU with this one's, itself included
     int tuned_threads = 0;
     int tuned_blocks_per_sm = 0;  // resident blocks per SM of the persistent launch (0: occupancy limit)
     cudaStream_t cap_stream = nullptr;
@@ -179,11 +180,20 @@ sbt_status cuda_fail(sbt_handle* h, cudaError_t e, const char* where)
     return fail(h, SBT_ERR_CUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 
-int default_threads(const sbt_handle* h, bool batched)
+// Threads of a search block: the configured number, for the batched launch
+// the autotuned one, else by the number of events.  While every event has a
+// block on the GPU at once, the call takes as long as the steps of its largest
+// event, and more warps shorten a step; beyond that the resident events count.
+// Two blocks of 512 fit an SM (64 registers), eight of 256, sixteen of 128 (32
+// registers).  Search, us at 512 / 256 / 128 threads: one event 230 / 251 /
+// 263, 100 events 336 / 402 / 574, 500 events 481 / 426 / 600, 1000 events
+// 960 / 531 / 693, 16000 events - / 6376 / 5397.
+int default_threads(const sbt_handle* h, bool batched, int64_t n_events)
 {
     if (h->cfg.threads_per_block) return h->cfg.threads_per_block;
     if (batched && h->tuned_threads) return h->tuned_threads;
-    return 128;
+    const int64_t events = n_events * h->concurrent;
+    return events <= 2 * (int64_t)h->sm_count ? 512 : events <= 8 * (int64_t)h->sm_count ? 256 : 128;
 }
 
 sbt_status check_inputs(sbt_handle* h, const float* x, const float* y, const float* z,
@@ -290,7 +300,11 @@ namespace sbt {
 
 const DevConfig& handle_device_config(const sbt_handle* h) { return h->C; }
 
-int handle_plain_threads(const sbt_handle* h) { return default_threads(h, false); }
+int handle_plain_threads(const sbt_handle* h, int64_t n_events) { return default_threads(h, false, n_events); }
+
+int handle_configured_threads(const sbt_handle* h) { return h->cfg.threads_per_block; }
+
+void handle_set_concurrent(sbt_handle* h, int handles) { h->concurrent = handles; }
 
 void handle_set_error(sbt_handle* h, const std::string& msg) { h->err = msg; }
 
@@ -380,7 +394,7 @@ sbt_status sbt_create(const sbt_geometry* geometry, const sbt_config* cfg, sbt_h
         delete h;
         return SBT_ERR_CUDA;
     }
-    if (sort_smem_bytes(h->C.nmax) > (size_t)max_optin || smem_bytes(h->C.nmax, 256, h->C.M) > (size_t)max_optin) {
+    if (sort_smem_bytes(h->C.nmax) > (size_t)max_optin || smem_bytes(h->C.nmax, 512, h->C.M) > (size_t)max_optin) {
         g_create_error = "max_hits_per_event exceeds shared memory";
         if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
         delete h;
@@ -434,7 +448,7 @@ sbt_status sbt_reconstruct(sbt_handle* h, const float* x, const float* y, const 
     carve_work(h->plain_arena.base, n_hits, n_events, &W);
     Inputs in = make_inputs(x, y, z, module, event_offsets, n_events, n_hits);
     e = launch_sort(h->C, in, O, s);
-    if (e == cudaSuccess) e = launch_plain(h->C, in, O, W, S, *out, default_threads(h, false), s);
+    if (e == cudaSuccess) e = launch_plain(h->C, in, O, W, S, *out, default_threads(h, false, n_events), s);
     if (e == cudaSuccess) e = launch_finish(h->C, in, S, *out, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "plain launch");
     h->launches_last = n_events > 0 ? 5 : 2;
@@ -449,7 +463,7 @@ sbt_status sbt_reconstruct_batched(sbt_handle* h, const float* x, const float* y
     sbt_status st = check_inputs(h, x, y, z, module, event_offsets, n_events, n_hits, out);
     if (st != SBT_OK || !out) return st != SBT_OK ? st : SBT_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    const int threads = default_threads(h, true);
+    const int threads = default_threads(h, true, n_events);
     const int blocks = persistent_blocks(h, threads);
     Staging S;
     Work W;
@@ -564,7 +578,7 @@ sbt_status sbt_reconstruct_host(sbt_handle* h, const float* x, const float* y, c
     if (e != cudaSuccess) return cuda_fail(h, e, "host-path allocation");
     Carver c1(h->host_arena.base);
     layout(c1, &dx, &dy, &dz, &dm, &doff, &dto, &dho, &dth, &dpar, &dchi, &dndof, &dstat, &dcnt, &drun);
-    const int threads = default_threads(h, true);
+    const int threads = default_threads(h, true, n_events);
     const int blocks = persistent_blocks(h, threads);
     Staging S;
     Work W;
@@ -870,7 +884,7 @@ sbt_status sbt_profile_batched(sbt_handle* h, const float* x, const float* y, co
     sbt_status st = check_inputs(h, x, y, z, module, event_offsets, n_events, n_hits, out);
     if (st != SBT_OK || !out || !ms || reps < 1) return st != SBT_OK ? st : fail(h, SBT_ERR_ARG, "bad argument");
     cudaStream_t s = (cudaStream_t)stream;
-    const int threads = default_threads(h, true);
+    const int threads = default_threads(h, true, n_events);
     const int blocks = persistent_blocks(h, threads);
     Staging S;
     Work W;

@@ -149,7 +149,11 @@ size_t adjoint_partial_entries(int M, int blocks);
 
 // Handle accessors for translation units that cannot see the handle type.
 const DevConfig& handle_device_config(const sbt_handle* h);
-int handle_plain_threads(const sbt_handle* h);
+int handle_plain_threads(const sbt_handle* h, int64_t n_events);
+int handle_configured_threads(const sbt_handle* h);
+// How many handles launch at the same time (the serving slots): their events
+// share the GPU, which decides the block size.
+void handle_set_concurrent(sbt_handle* h, int handles);
 void handle_set_error(sbt_handle* h, const std::string& msg);
 void handle_set_launches(sbt_handle* h, int launches);
 // Workspaces the handle outgrows are kept until sbt_destroy instead of freed

@@ -174,7 +174,7 @@ extern "C" sbt_status sbt_reconstruct_noalloc(sbt_handle* h, const float* x, con
     cudaStream_t s = (cudaStream_t)stream;
     const DevConfig& C = handle_device_config(h);
     e = launch_sort(C, in, O, s);
-    if (e == cudaSuccess) e = launch_plain(C, in, O, W, S, *out, handle_plain_threads(h), s);
+    if (e == cudaSuccess) e = launch_plain(C, in, O, W, S, *out, handle_plain_threads(h, n_events), s);
     if (e == cudaSuccess) e = launch_finish(C, in, S, *out, s);
     if (e != cudaSuccess) {
         handle_set_error(h, std::string("noalloc launch: ") + cudaGetErrorString(e));

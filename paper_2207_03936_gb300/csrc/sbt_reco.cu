@@ -1159,12 +1159,15 @@ __device__ void run_event(const DevConfig& C, const Inputs& in, const Sorted& O,
 
 // Residency of the search: the kernel waits on load latency, so throughput
 // follows the number of resident events; the compiler is asked for a
-// register count that lets 2048 threads (32 blocks of 64) share an SM.
-constexpr int kSearchThreadsPerSM = 2048;
+// register count that lets 2048 threads share an SM (16 blocks of 128, 16000
+// uneven events: 5.40 ms; 1536 threads 5.94, 1024 threads 6.65).  Blocks of 512
+// run calls of a few events, where a step's length counts: 64 registers, no
+// spills (one event 251 us at 256 threads and 32 registers, 229 us at 64).
+constexpr int search_blocks_per_sm(int threads) { return (threads == 512 ? 1024 : 2048) / threads; }
 
 // One block per event.
 template <int NT, class HS, class GEO>
-__global__ void __launch_bounds__(NT, kSearchThreadsPerSM / NT) k_search_plain(DevConfig C, Inputs in, Sorted O, Work W,
+__global__ void __launch_bounds__(NT, search_blocks_per_sm(NT)) k_search_plain(DevConfig C, Inputs in, Sorted O, Work W,
                                                       Staging G, sbt_tracks out)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1179,7 +1182,7 @@ __global__ void __launch_bounds__(NT, kSearchThreadsPerSM / NT) k_search_plain(D
 // alternating from both ends of G.order (largest first), and reuses its own
 // scratch region.
 template <int NT, class HS, class GEO>
-__global__ void __launch_bounds__(NT, kSearchThreadsPerSM / NT) k_search_persistent(DevConfig C, Inputs in, Sorted O, Work W,
+__global__ void __launch_bounds__(NT, search_blocks_per_sm(NT)) k_search_persistent(DevConfig C, Inputs in, Sorted O, Work W,
                                                            Staging G, sbt_tracks out)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1525,6 +1528,7 @@ cudaError_t launch_plain(const DevConfig& C, const Inputs& in, const Sorted& O, 
         case 64: return C.h16 ? plain_nt<64, HitsF16>(C, in, O, W, S, out, stream) : plain_nt<64, HitsF32>(C, in, O, W, S, out, stream);
         case 128: return C.h16 ? plain_nt<128, HitsF16>(C, in, O, W, S, out, stream) : plain_nt<128, HitsF32>(C, in, O, W, S, out, stream);
         case 256: return C.h16 ? plain_nt<256, HitsF16>(C, in, O, W, S, out, stream) : plain_nt<256, HitsF32>(C, in, O, W, S, out, stream);
+        case 512: return C.h16 ? plain_nt<512, HitsF16>(C, in, O, W, S, out, stream) : plain_nt<512, HitsF32>(C, in, O, W, S, out, stream);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -1561,6 +1565,7 @@ int persistent_blocks_per_sm(const DevConfig& C, int threads)
         case 64: return C.h16 ? occupancy_nt<64, HitsF16>(C) : occupancy_nt<64, HitsF32>(C);
         case 128: return C.h16 ? occupancy_nt<128, HitsF16>(C) : occupancy_nt<128, HitsF32>(C);
         case 256: return C.h16 ? occupancy_nt<256, HitsF16>(C) : occupancy_nt<256, HitsF32>(C);
+        case 512: return C.h16 ? occupancy_nt<512, HitsF16>(C) : occupancy_nt<512, HitsF32>(C);
         default: return 0;
     }
 }
@@ -1595,6 +1600,7 @@ cudaError_t launch_persistent(const DevConfig& C, const Inputs& in, const Sorted
         case 64: return C.h16 ? persistent_nt<64, HitsF16>(C, in, O, W, S, out, blocks, stream) : persistent_nt<64, HitsF32>(C, in, O, W, S, out, blocks, stream);
         case 128: return C.h16 ? persistent_nt<128, HitsF16>(C, in, O, W, S, out, blocks, stream) : persistent_nt<128, HitsF32>(C, in, O, W, S, out, blocks, stream);
         case 256: return C.h16 ? persistent_nt<256, HitsF16>(C, in, O, W, S, out, blocks, stream) : persistent_nt<256, HitsF32>(C, in, O, W, S, out, blocks, stream);
+        case 512: return C.h16 ? persistent_nt<512, HitsF16>(C, in, O, W, S, out, blocks, stream) : persistent_nt<512, HitsF32>(C, in, O, W, S, out, blocks, stream);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -488,7 +488,7 @@ sbt_status sbt_server_create(sbt_handle* h, int64_t memory_budget_bytes, int32_t
     cfg.hit_sigma = C.sigma;
     cfg.max_hits_per_event = C.nmax;
     cfg.max_forming_tracks = C.fcap;
-    cfg.threads_per_block = sbt::handle_plain_threads(h);
+    cfg.threads_per_block = sbt::handle_configured_threads(h);
     cfg.gec_max_hits = C.gec;
     cfg.fp16_hits = C.h16;
     for (int i = 0; i < max_streams && e == cudaSuccess; i++) {
@@ -516,7 +516,10 @@ sbt_status sbt_server_create(sbt_handle* h, int64_t memory_budget_bytes, int32_t
         delete S;
         return SBT_ERR_CUDA;
     }
-    for (auto& sl : S->slots) sbt::handle_defer_frees(sl->h);
+    for (auto& sl : S->slots) {
+        sbt::handle_defer_frees(sl->h);
+        sbt::handle_set_concurrent(sl->h, max_streams);
+    }
     S->allocs0 = g_allocs.load();
     S->launcher = std::thread(launcher_loop, S);
     S->harvester = std::thread(harvester_loop, S);
