@@ -144,7 +144,7 @@ __device__ __forceinline__ void fit_line(int n, Get get, float sigma, float* par
 // ------------------------------------------------------- shared layout ---
 
 enum Misc {
-    kErr = 0, kNFin = 1, kNTl = 2, kEvent = 3, kCMask = 4, kCnt0 = 5, kCnt1 = 6, kNew = 7, kWork = 8, kList = 9,
+    kErr = 0, kNFin = 1, kNTl = 2, kEvent = 3, kCMask = 4, kCnt0 = 5, kCnt1 = 6, kWork = 7, kNew = 8, kList = 9,
     kNOuter = 10, kMiscN = 12
 };
 
@@ -835,7 +835,8 @@ __device__ __forceinline__ void follow_and_claim(const DevConfig& C, const Smem&
 //   P1  seeding, kSeedLanes lanes per middle hit, and following of the forming
 //       tracks to t = s+3 with claims: a warp keeps its new seeds in its lanes
 //       and fills the other lanes with old tracks from a shared counter, so
-//       its following rounds are dense;
+//       its following rounds are dense; it leaves after the round that found
+//       the counter used up (an empty round costs a few hundred clocks);
 //   P2  resolution of the claims, flags, termination.
 // Claims carry a tag (64 - t) << 48 above (scatter bits, track key), so a
 // claim of an earlier step always compares larger than one of the current
@@ -895,8 +896,7 @@ __device__ bool search_stage(const DevConfig& C, const Region<HS>& R, const Smem
         int na = 0, nc = -1, nb = 0;  // this lane's new seed
         int i0 = (tid >> 5) * kSeedGroups, batch = 0;
         for (;;) {
-            const bool seeding = i0 < nl;
-            if (seeding) {
+            if (i0 < nl) {
                 const int i = i0 + lane / kSeedLanes;
                 const int c = i < nl ? (int)list[i] : -1;
                 const unsigned long long best = seed_group<G>(C, S, R, s, c, outer, nu, sq_seed);
@@ -910,17 +910,18 @@ __device__ bool search_stage(const DevConfig& C, const Region<HS>& R, const Smem
                 if (++batch < kSeedLanes && i0 < nl) continue;
                 batch = 0;
             }
-            // following: this warp's new seeds, and old tracks in the other lanes
-            const unsigned idle = __ballot_sync(0xFFFFFFFFu, nc < 0);
-            int base = nold;
-            if (follow && idle) {
-                if (lane == 0) base = atomicAdd(&misc[kWork], __popc(idle));
-                base = __shfl_sync(0xFFFFFFFFu, base, 0);
-            }
-            int slot = base + __popc(idle & ((1u << lane) - 1u));
+            // following: this warp's new seeds, and old tracks in the other
+            // lanes; one atomic instruction numbers both
+            const unsigned found = __ballot_sync(0xFFFFFFFFu, nc >= 0);
+            int base = 0;
+            if (lane < 2 && (lane == 0 ? follow : found != 0))
+                base = atomicAdd(&misc[kWork + lane], __popc(lane == 0 ? ~found : found));
+            const int taken = follow ? __shfl_sync(0xFFFFFFFFu, base, 0) : nold;
+            const int fresh = nold + __shfl_sync(0xFFFFFFFFu, base, 1);
+            const unsigned below = (1u << lane) - 1u;
+            int slot = nc >= 0 ? fresh + __popc(found & below) : taken + __popc(~found & below);
             FTrack T;
             if (nc >= 0) {
-                slot = nold + atomicAdd(&misc[kNew], 1);
                 T = make_track(na, nc, nb, nc, 3, 0);
                 if (slot >= cap) {
                     misc[kErr] = SBT_ERR_CAPACITY;
@@ -936,7 +937,7 @@ __device__ bool search_stage(const DevConfig& C, const Region<HS>& R, const Smem
                 Fc[slot] = T;
             }
             nc = -1;
-            if (!seeding && base + __popc(idle) >= nold) break;
+            if (i0 >= nl && taken + 32 - __popc(found) >= nold) break;
         }
         __syncthreads();
         if (misc[kErr]) return false;
