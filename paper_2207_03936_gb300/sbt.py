@@ -443,17 +443,20 @@ class Server:
         if st == SBT_ERR_TIMEOUT:
             return []
         _check(st)
+
+        def copy(address, count, dtype):
+            # a view of an array type per length costs more than the copy
+            # (ctypes builds a class for each)
+            raw = ctypes.string_at(address, 4 * count) if count else b""
+            return np.frombuffer(raw, dtype).copy()
+
         out = []
         for r in buf[:n.value]:
             T = r.n_tracks
-            ho = np.ctypeslib.as_array((ctypes.c_int32 * (T + 1)).from_address(r.hit_offsets)).copy()
-            H = int(ho[-1])
-            th = (np.ctypeslib.as_array((ctypes.c_int32 * H).from_address(r.track_hits)).copy()
-                  if H else np.zeros(0, np.int32))
-            pr = (np.ctypeslib.as_array((ctypes.c_float * (4 * T)).from_address(r.params)).copy()
-                  if T else np.zeros(0, np.float32))
-            c2 = (np.ctypeslib.as_array((ctypes.c_float * T).from_address(r.chi2)).copy()
-                  if T else np.zeros(0, np.float32))
+            ho = copy(r.hit_offsets, T + 1, np.int32)
+            th = copy(r.track_hits, int(ho[-1]), np.int32)
+            pr = copy(r.params, 4 * T, np.float32)
+            c2 = copy(r.chi2, T, np.float32)
             out.append(ServedResult(r.request_id, r.status, ho, th, pr.reshape(T, 4), c2, r.latency_s))
             self.L.sbt_server_release(self.s, r.request_id)
         return out
