@@ -1277,79 +1277,6 @@ __global__ void __launch_bounds__(1024) k_scan(Inputs in, Staging G, sbt_tracks 
     }
 }
 
-// Least-squares fit of one track from its n staged hit records (src), with
-// its hit list written on the way (th: batch input indices): sums in hit
-// order, every operation rounded as in fit_line.  The first pass loads the
-// records four at a time (independent loads in flight) and keeps the
-// coordinates of the first kFitStash in shared memory (stash: this thread's
-// column of a [kFitStash][kFitThreads] float3 array, conflict-free); the two
-// centred passes read them there and re-read only the others.
-constexpr int kFitThreads = 256;
-constexpr int kFitStash = 16;
-
-__device__ __forceinline__ void fit_staged(int n, const float4* src, int32_t* th, float3* stash, float sigma,
-                                           float* params, float* chi2)
-{
-    float sx = 0.0f, sy = 0.0f, sz = 0.0f;
-    for (int i0 = 0; i0 < n; i0 += 4) {
-        float4 v[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++)
-            if (i0 + u < n) v[u] = src[i0 + u];
-#pragma unroll
-        for (int u = 0; u < 4; u++)
-            if (i0 + u < n) {
-                th[i0 + u] = __float_as_int(v[u].w);
-                sx = __fadd_rn(sx, v[u].x);
-                sy = __fadd_rn(sy, v[u].y);
-                sz = __fadd_rn(sz, v[u].z);
-                if (i0 + u < kFitStash) stash[(i0 + u) * kFitThreads] = make_float3(v[u].x, v[u].y, v[u].z);
-            }
-    }
-    const int ns = min(n, kFitStash);
-    const float nf = (float)n;
-    const float xm = __fdiv_rn(sx, nf), ym = __fdiv_rn(sy, nf), zm = __fdiv_rn(sz, nf);
-    float szz = 0.0f, szx = 0.0f, szy = 0.0f;
-    auto moments = [&](float x, float y, float z) {
-        const float dz = __fsub_rn(z, zm);
-        szz = __fadd_rn(szz, __fmul_rn(dz, dz));
-        szx = __fadd_rn(szx, __fmul_rn(dz, __fsub_rn(x, xm)));
-        szy = __fadd_rn(szy, __fmul_rn(dz, __fsub_rn(y, ym)));
-    };
-#pragma unroll 4
-    for (int i = 0; i < ns; i++) {
-        const float3 q = stash[i * kFitThreads];
-        moments(q.x, q.y, q.z);
-    }
-    for (int i = kFitStash; i < n; i++) {
-        const float4 q = src[i];
-        moments(q.x, q.y, q.z);
-    }
-    const float tx = __fdiv_rn(szx, szz);
-    const float ty = __fdiv_rn(szy, szz);
-    float s = 0.0f;
-    auto resid = [&](float x, float y, float z) {
-        const float dz = __fsub_rn(z, zm);
-        const float rx = __fsub_rn(__fsub_rn(x, xm), __fmul_rn(tx, dz));
-        const float ry = __fsub_rn(__fsub_rn(y, ym), __fmul_rn(ty, dz));
-        s = __fadd_rn(s, __fadd_rn(__fmul_rn(rx, rx), __fmul_rn(ry, ry)));
-    };
-#pragma unroll 4
-    for (int i = 0; i < ns; i++) {
-        const float3 q = stash[i * kFitThreads];
-        resid(q.x, q.y, q.z);
-    }
-    for (int i = kFitStash; i < n; i++) {
-        const float4 q = src[i];
-        resid(q.x, q.y, q.z);
-    }
-    params[0] = __fsub_rn(xm, __fmul_rn(tx, zm));
-    params[1] = __fsub_rn(ym, __fmul_rn(ty, zm));
-    params[2] = tx;
-    params[3] = ty;
-    *chi2 = __fdiv_rn(s, __fmul_rn(sigma, sigma));
-}
-
 // Output (section "Results", data consolidation), one block per event: the
 // canonical order of the event's tracks by smallest input hit index and
 // their CSR starts; the hit lists and fits follow in k_fit.  A track's rank
@@ -1424,22 +1351,116 @@ __global__ void __launch_bounds__(kOutputThreads) k_output(DevConfig C, Inputs i
 // Hit lists and least-squares fits of the canonical tracks, one thread per
 // track of the batch, in canonical order (a warp's hit lists and parameters
 // are contiguous in the output): the tracks of the events the output kernel
-// wrote, G.queue[1] of them.
-__global__ void __launch_bounds__(kFitThreads) k_fit(DevConfig C, Staging G, sbt_tracks out)
+// wrote, G.queue[1] of them.  A warp first copies its 32 tracks, lanes over the
+// hits of one track at a time, four tracks in flight: the staged records come
+// in coalesced, the hit lists go out coalesced, and the coordinates of the first
+// kFitRows hits land in shared memory, one column per track, where every lane
+// then reads its own without conflicts (33 words a row).  With each lane
+// loading its own track's records and storing its own hit list, every lane was
+// an L1 wavefront of its own (two a hit, the LSU data pipe 74% busy).  The sums
+// run in hit order, every operation rounded as in fit_line.
+constexpr int kFitThreads = 128;
+constexpr int kFitRows = 16;
+constexpr int kFitAhead = 4;
+// Six blocks an SM (80 registers, 25 KB a block) hold enough loads in flight:
+// output step of 16000 uneven events 798 -> 660 us; at four blocks with 24 rows
+// 744, five with 20 rows 687, eight (64 registers) 893; half as many tracks in
+// flight 960.
+constexpr int kFitBlocksPerSM = 6;
+
+__global__ void __launch_bounds__(kFitThreads, kFitBlocksPerSM) k_fit(DevConfig C, Staging G, sbt_tracks out)
 {
-    __shared__ float3 stash[kFitStash * kFitThreads];
+    __shared__ float rows[kFitThreads / 32][3][kFitRows][33];
+    const int lane = threadIdx.x & 31;
+    float(*col)[kFitRows][33] = rows[threadIdx.x >> 5];
     const int T = G.queue[1];
-    for (int g = blockIdx.x * kFitThreads + threadIdx.x; g < T; g += gridDim.x * kFitThreads) {
-        const uint2 f = G.tfit[g];
+    const bool wide = ((uintptr_t)out.params & 15) == 0;
+    for (int64_t g0 = (int64_t)blockIdx.x * kFitThreads + (threadIdx.x & ~31); g0 < T;
+         g0 += (int64_t)gridDim.x * kFitThreads) {
+        const int64_t g = g0 + lane;
+        const uint2 f = g < T ? G.tfit[g] : make_uint2(0u, 0u);
         const int n = (int)f.y;
-        float p[4], chi2;
-        fit_staged(n, G.hits + f.x, out.track_hits + out.hit_offsets[g], stash + threadIdx.x, C.sigma, p, &chi2);
-        out.params[4 * (int64_t)g + 0] = p[0];
-        out.params[4 * (int64_t)g + 1] = p[1];
-        out.params[4 * (int64_t)g + 2] = p[2];
-        out.params[4 * (int64_t)g + 3] = p[3];
-        out.chi2[g] = chi2;
-        out.ndof[g] = 2 * n - 4;
+        const int to = g < T ? out.hit_offsets[g] : 0;
+        // half a warp per track: hits 0-15 of two tracks, then 16-31 where there are any
+        const int half = lane >> 4, j0 = lane & 15;
+        for (int k0 = 0; k0 < 32; k0 += 2 * kFitAhead) {
+            float4 v[kFitAhead], w[kFitAhead];
+            int nk[kFitAhead], tk[kFitAhead];
+#pragma unroll
+            for (int u = 0; u < kFitAhead; u++) {
+                const int k = k0 + 2 * u + half;
+                nk[u] = __shfl_sync(0xFFFFFFFFu, n, k);
+                tk[u] = __shfl_sync(0xFFFFFFFFu, to, k);
+                const float4* sk = G.hits + (__shfl_sync(0xFFFFFFFFu, f.x, k) + (uint32_t)j0);
+                if (j0 < nk[u]) v[u] = sk[0];
+                if (j0 + 16 < nk[u]) w[u] = sk[16];
+            }
+            auto keep = [&](float4 c, int j, int u) {
+                out.track_hits[tk[u] + j] = __float_as_int(c.w);
+                if (j < kFitRows) {
+                    const int k = k0 + 2 * u + half;
+                    col[0][j][k] = c.x;
+                    col[1][j][k] = c.y;
+                    col[2][j][k] = c.z;
+                }
+            };
+#pragma unroll
+            for (int u = 0; u < kFitAhead; u++) {
+                if (j0 < nk[u]) keep(v[u], j0, u);
+                if (j0 + 16 < nk[u]) keep(w[u], j0 + 16, u);
+            }
+        }
+        __syncwarp();
+        // hits past the rows, and hit lists past a warp's lanes
+        const float4* src = G.hits + f.x;
+        for (int j = 32; j < n; j++) out.track_hits[to + j] = __float_as_int(src[j].w);
+        const int ns = min(n, kFitRows);
+        auto each = [&](auto use) {
+#pragma unroll 4
+            for (int j = 0; j < ns; j++) use(col[0][j][lane], col[1][j][lane], col[2][j][lane]);
+            for (int j = kFitRows; j < n; j++) {
+                const float4 q = src[j];
+                use(q.x, q.y, q.z);
+            }
+        };
+        if (n > 0) {
+            float sx = 0.0f, sy = 0.0f, sz = 0.0f;
+            each([&](float x, float y, float z) {
+                sx = __fadd_rn(sx, x);
+                sy = __fadd_rn(sy, y);
+                sz = __fadd_rn(sz, z);
+            });
+            const float nf = (float)n;
+            const float xm = __fdiv_rn(sx, nf), ym = __fdiv_rn(sy, nf), zm = __fdiv_rn(sz, nf);
+            float szz = 0.0f, szx = 0.0f, szy = 0.0f;
+            each([&](float x, float y, float z) {
+                const float dz = __fsub_rn(z, zm);
+                szz = __fadd_rn(szz, __fmul_rn(dz, dz));
+                szx = __fadd_rn(szx, __fmul_rn(dz, __fsub_rn(x, xm)));
+                szy = __fadd_rn(szy, __fmul_rn(dz, __fsub_rn(y, ym)));
+            });
+            const float tx = __fdiv_rn(szx, szz);
+            const float ty = __fdiv_rn(szy, szz);
+            float s = 0.0f;
+            each([&](float x, float y, float z) {
+                const float dz = __fsub_rn(z, zm);
+                const float rx = __fsub_rn(__fsub_rn(x, xm), __fmul_rn(tx, dz));
+                const float ry = __fsub_rn(__fsub_rn(y, ym), __fmul_rn(ty, dz));
+                s = __fadd_rn(s, __fadd_rn(__fmul_rn(rx, rx), __fmul_rn(ry, ry)));
+            });
+            const float4 p = make_float4(__fsub_rn(xm, __fmul_rn(tx, zm)), __fsub_rn(ym, __fmul_rn(ty, zm)), tx, ty);
+            if (wide) {
+                ((float4*)out.params)[g] = p;
+            } else {
+                out.params[4 * g + 0] = p.x;
+                out.params[4 * g + 1] = p.y;
+                out.params[4 * g + 2] = p.z;
+                out.params[4 * g + 3] = p.w;
+            }
+            out.chi2[g] = __fdiv_rn(s, __fmul_rn(C.sigma, C.sigma));
+            out.ndof[g] = 2 * n - 4;
+        }
+        __syncwarp();
     }
 }
 

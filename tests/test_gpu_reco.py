@@ -436,6 +436,24 @@ def test_output_capacity_overflow_writes_the_fitting_events_only(sbt, handle):
     assert np.array_equal(nd[:tw], full["ndof"][:tw]) and (nd[tw:] == -7).all()
 
 
+@pytest.mark.parametrize("batched", [False, True])
+def test_fit_kernel_track_lengths_and_unaligned_params(sbt, handle, batched):
+    """Tracks around the fit kernel's row limit, its half warps and a warp's
+    lanes (15 to 52 hits), 1 to 67 tracks (fewer and more than a warp takes),
+    and a params array that starts on no 16-byte boundary."""
+    for lengths in ([15], [16, 17], [31, 32, 33, 34], [52, 3, 48, 16], [20] * 67):
+        parts = [line_hits(8.0 * np.cos(p), 8.0 * np.sin(p), 0.02 * np.cos(p), 0.02 * np.sin(p), range(52 - n, 52))
+                 for n, p in zip(lengths, np.linspace(0.1, 6.2, len(lengths)))]
+        x, y, z, m, _ = assemble(parts, 11)
+        ev = arrays(x, y, z, m)
+        ref = oracle_of(ev)
+        assert sorted(np.diff(ref.hit_offsets)) == sorted(lengths)
+        out = sbt.TrackOutput.allocate(1, ev.n_hits)
+        out.params = torch.zeros(out.params.numel() + 1, dtype=torch.float32, device="cuda")[1:]
+        fn = sbt.sbt_reconstruct_batched if batched else sbt.sbt_reconstruct
+        assert_same(fn(handle, *to_dev(ev), out=out).compact(), ref)
+
+
 def test_repeat_runs_are_identical(sbt, handle):
     ev = synth.make_events(2, 200, workers=1)
     a = run_gpu(sbt, handle, ev, True)
