@@ -254,7 +254,8 @@ sbt_status sbt_debug_phi16(const float* x, const float* y, int32_t n, uint16_t* 
  * timing each kernel with CUDA events on `stream`, and writes the mean
  * milliseconds per launch to ms[5] (host): ordering kernel, sort kernel,
  * persistent search kernel, scan, output (the output kernel's canonical
- * order and CSR starts, then the fit kernel's hit lists and fits).
+ * order and CSR starts, then the fit kernel's hit lists and fits; a batch of
+ * at most 64 events runs scan and output as one kernel, timed as output).
  * Synchronous.
  */
 sbt_status sbt_profile_batched(sbt_handle* h, const float* x, const float* y, const float* z,

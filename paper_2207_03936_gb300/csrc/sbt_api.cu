@@ -451,7 +451,7 @@ sbt_status sbt_reconstruct(sbt_handle* h, const float* x, const float* y, const 
     if (e == cudaSuccess) e = launch_plain(h->C, in, O, W, S, *out, default_threads(h, false, n_events), s);
     if (e == cudaSuccess) e = launch_finish(h->C, in, S, *out, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "plain launch");
-    h->launches_last = n_events > 0 ? 5 : 2;
+    h->launches_last = n_events > 0 ? 2 + finish_launches(n_events) : 2;
     return SBT_OK;
 }
 
@@ -515,7 +515,7 @@ sbt_status sbt_reconstruct_batched(sbt_handle* h, const float* x, const float* y
     }
     cudaError_t e = cudaGraphLaunch(h->exec, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "graph launch");
-    h->launches_last = n_events > 0 ? 6 : 2;
+    h->launches_last = n_events > 0 ? 3 + finish_launches(n_events) : 2;
     return SBT_OK;
 }
 
@@ -725,7 +725,7 @@ sbt_status sbt_reconstruct_host(sbt_handle* h, const float* x, const float* y, c
     oh->counts[1] = (int32_t)HH;
     oh->counts[2] = cap_ok ? SBT_OK : SBT_ERR_CAPACITY;
     oh->counts[3] = (int32_t)failed;
-    h->launches_last = C * 7;
+    h->launches_last = C > 1 || n_events == 0 ? C * 7 : 4 + finish_launches(n_events);
     return SBT_OK;
 }
 
@@ -912,9 +912,10 @@ sbt_status sbt_profile_batched(sbt_handle* h, const float* x, const float* y, co
         if (e == cudaSuccess && n_events > 0)
             e = launch_persistent(h->C, in, O, W, S, *out, threads, std::min(blocks, n_events), s);
         if (e == cudaSuccess) e = cudaEventRecord(ev[3], s);
-        if (e == cudaSuccess) e = launch_scan(in, S, *out, s);
+        const bool one = n_events > 0 && finish_launches(n_events) == 1;  // its time counts as output
+        if (e == cudaSuccess && !one) e = launch_scan(in, S, *out, s);
         if (e == cudaSuccess) e = cudaEventRecord(ev[4], s);
-        if (e == cudaSuccess) e = launch_output(h->C, in, S, *out, s);
+        if (e == cudaSuccess) e = one ? launch_finish(h->C, in, S, *out, s) : launch_output(h->C, in, S, *out, s);
         if (e == cudaSuccess) e = cudaEventRecord(ev[5], s);
         if (e == cudaSuccess) e = cudaEventSynchronize(ev[5]);
         for (int k = 0; k < 5 && e == cudaSuccess; k++) {

@@ -115,7 +115,9 @@ cudaError_t launch_order(const Inputs& in, const Staging& S, cudaStream_t stream
 cudaError_t launch_persistent(const DevConfig& C, const Inputs& in, const Sorted& O, const Work& W,
                               const Staging& S, const sbt_tracks& out, int threads, int blocks,
                               cudaStream_t stream);
-// Scan of the per-event counts, then the output kernel (CSR hit lists and fits).
+// Scan of the per-event counts, order and fits of the tracks: one kernel for a
+// small batch, else launch_scan and launch_output (finish_launches kernels).
+int finish_launches(int n_events);
 cudaError_t launch_finish(const DevConfig& C, const Inputs& in, const Staging& S,
                           const sbt_tracks& out, cudaStream_t stream);
 cudaError_t launch_scan(const Inputs& in, const Staging& S, const sbt_tracks& out,

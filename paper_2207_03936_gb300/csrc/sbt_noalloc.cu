@@ -180,6 +180,6 @@ extern "C" sbt_status sbt_reconstruct_noalloc(sbt_handle* h, const float* x, con
         handle_set_error(h, std::string("noalloc launch: ") + cudaGetErrorString(e));
         return SBT_ERR_CUDA;
     }
-    handle_set_launches(h, n_events > 0 ? 5 : 2);
+    handle_set_launches(h, n_events > 0 ? 2 + finish_launches(n_events) : 2);
     return SBT_OK;
 }

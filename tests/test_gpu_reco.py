@@ -454,6 +454,35 @@ def test_fit_kernel_track_lengths_and_unaligned_params(sbt, handle, batched):
         assert_same(fn(handle, *to_dev(ev), out=out).compact(), ref)
 
 
+@pytest.mark.parametrize("events", [1, 63, 64, 65])
+def test_last_kernel_of_small_batches(sbt, handle, events):
+    """Batches up to 64 events end in one kernel (counts of the events before,
+    order, fits), larger ones in three: results, failed events among them, and
+    the fitting events of a batch whose outputs are too small."""
+    ev = synth.make_events(2, events, seed=3, workers=1)
+    if events > 1:
+        ev.module = ev.module.copy()
+        ev.module[int(ev.event_offsets[events // 2])] = 77       # one failed event
+    ref = oracle_of(ev)
+    for batched in (False, True):
+        g = run_gpu(sbt, handle, ev, batched)
+        assert int(g["counts"][3]) == int(events > 1)
+        assert_same(g, ref)
+    for cap in (ref.n_tracks - 1, ref.n_tracks // 2, 0):
+        fit = int(np.searchsorted(ref.track_offsets, cap, side="right")) - 1   # events that fit whole
+        tw = int(ref.track_offsets[fit])
+        hw = int(ref.hit_offsets[tw])
+        out = sbt.TrackOutput.allocate(ev.n_events, ev.n_hits, cap_tracks=cap)
+        out.track_hits.fill_(-7)
+        out.chi2.fill_(-7.0)
+        sbt.sbt_reconstruct(handle, *to_dev(ev), out=out)
+        assert out.counts.tolist()[:3] == [ref.n_tracks, len(ref.track_hits), sbt.SBT_ERR_CAPACITY]
+        assert np.array_equal(out.track_offsets.cpu().numpy(), ref.track_offsets)
+        th, chi = out.track_hits.cpu().numpy(), out.chi2.cpu().numpy()
+        assert np.array_equal(th[:hw], ref.track_hits[:hw]) and (th[hw:] == -7).all()
+        assert np.array_equal(chi[:tw].view(np.uint32), ref.chi2[:tw].view(np.uint32)) and (chi[tw:] == -7).all()
+
+
 def test_repeat_runs_are_identical(sbt, handle):
     ev = synth.make_events(2, 200, workers=1)
     a = run_gpu(sbt, handle, ev, True)
