@@ -110,7 +110,7 @@ size_t carve_sorted(void* base, int64_t n_hits, int64_t n_events, int M, Sorted*
     Carver c(base);
     Sorted o;
     o.coords = c.take<float4>(n_hits);
-    o.phi = c.take<uint16_t>(n_hits);
+    o.index = c.take<uint16_t>(n_hits);
     o.bucket = c.take<uint16_t>(n_events * (M << kBucketBits));
     o.modoff = c.take<int32_t>(n_events * (M + 1));
     o.status = c.take<int32_t>(n_events);

@@ -10,7 +10,10 @@
 namespace sbt {
 
 constexpr int kMaxModules = 64;
-constexpr int kBucketBits = 6;           // the sort's buckets: top bits of phi16 within a module
+// The sort's buckets, top bits of phi16 within a module: about one hit each, so
+// that a window's scan starts near its edge (search of 92 M hits 5.28 ms with 6
+// bits, 5.07 with 7).
+constexpr int kBucketBits = 7;
 constexpr int kMaxHitsPerEvent = 16384;  // the per-event sort runs in shared memory
 
 // Method constants and per-event capacities, passed to kernels by value.
@@ -57,9 +60,9 @@ inline int64_t forming_entries(int64_t hits, int64_t regions) { return 2 * (hits
 struct Sorted {
     float4* coords;   // (x, y, z, phi16 << 16 | event-local input index) by sorted position, or
                       // fp16 records
-    uint16_t* phi;    // phi16 by sorted position (fp16 records only)
+    uint16_t* index;  // event-local input index by sorted position (fp16 records only)
     uint16_t* bucket; // [n_events * (n_modules << kBucketBits)] event-local start of every
-                      // (module, phi16 >> 10): where a window's scan begins
+                      // (module, phi16 >> 9): where a window's scan begins
     int32_t* modoff;  // [n_events * (n_modules + 1)] event-local module offsets
     int32_t* status;  // [n_events] SBT_OK, SBT_ERR_ARG or SBT_ERR_CAPACITY after the sort
 };

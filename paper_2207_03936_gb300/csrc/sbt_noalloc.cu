@@ -28,7 +28,7 @@ constexpr size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 // Offsets of the workspace arrays (the Sorted, Work and Staging layouts for
 // kNoAllocMaxHits hits and kNoAllocMaxEvents events), each 256-byte aligned.
 struct Layout {
-    size_t coords, phi, bucket, modoff, status;
+    size_t coords, index, bucket, modoff, status;
     size_t list, prev, claim, ft, tracklets, tl_q, finals;
     size_t hits, tkey, tinfo, rinfo, tfit, ntracks, nhits, track_base, hit_base, order, queue, total;
 };
@@ -40,7 +40,7 @@ constexpr Layout make_layout()
     const int64_t TL = H + E + 1, FN = H / 3 + E + 1;
     size_t o = 0;
     L.coords = o;     o = align256(o + 16 * (size_t)H);
-    L.phi = o;        o = align256(o + 2 * (size_t)H);
+    L.index = o;       o = align256(o + 2 * (size_t)H);
     L.bucket = o;     o = align256(o + 2 * (size_t)E * (kMaxModules << kBucketBits));
     L.modoff = o;     o = align256(o + 4 * (size_t)E * (kMaxModules + 1));
     L.status = o;     o = align256(o + 4 * (size_t)E);
@@ -68,7 +68,7 @@ constexpr Layout make_layout()
 
 constexpr Layout kLayout = make_layout();
 
-// The workspace (about 82 MB).  In host code this name is only a host-side
+// The workspace (about 115 MB).  In host code this name is only a host-side
 // stand-in: its device address comes from cudaGetSymbolAddress below.
 __device__ __align__(256) unsigned char g_noalloc_workspace[kLayout.total];
 
@@ -135,7 +135,7 @@ extern "C" sbt_status sbt_reconstruct_noalloc(sbt_handle* h, const float* x, con
     const Layout& L = kLayout;
     Sorted O;
     O.coords = (float4*)(base + L.coords);
-    O.phi = (uint16_t*)(base + L.phi);
+    O.index = (uint16_t*)(base + L.index);
     O.bucket = (uint16_t*)(base + L.bucket);
     O.modoff = (int32_t*)(base + L.modoff);
     O.status = (int32_t*)(base + L.status);

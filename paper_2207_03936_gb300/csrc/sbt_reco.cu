@@ -6,8 +6,8 @@
 //      index) from one counting pass into (module, coarse phi) buckets and a
 //      sort inside each bucket, in shared memory (section "Sort by phi"); the
 //      sorted hits are written as AoS records (x, y, z, phi16 and input
-//      index: float4, or fp16 x, y, z and a 16-bit index with phi16 beside),
-//      with the start of every bucket;
+//      index: float4, or fp16 x, y, z and phi16 with the index beside), with
+//      the start of every bucket;
 //   2. k_search_*: for every module triplet (s, s+1, s+2): seeding over the unflagged
 //      middle hits, then following of every forming track to module s+3 with
 //      one-round claims on the hits, flags, and termination after two misses
@@ -195,74 +195,60 @@ __device__ __forceinline__ bool flagged(const Smem& S, int p) { return (S.flag[p
 __device__ __forceinline__ void set_flag(const Smem& S, int p) { atomicOr(&S.flag[p >> 5], 1u << (p & 31)); }
 
 // Storage of the sorted hits.  HitsF32: float4 (x, y, z, phi16 << 16 | input
-// index as int bits), 16 bytes: one load gives a window scan the key and the
-// position.  HitsF16: x, y, z rounded to fp16 (nearest even) and the input
-// index in 16 bits, 8 bytes (the paper's fp16 AoS storage of hit
-// coordinates), phi16 in an array of its own; every computation still runs in
-// fp32, on the rounded values.
+// index as int bits), 16 bytes.  HitsF16: x, y, z rounded to fp16 (nearest
+// even) and phi16, 8 bytes (the paper's fp16 AoS storage of hit coordinates),
+// the input index in an array of its own, which only the output reads; every
+// computation still runs in fp32, on the rounded values.  Either way one load
+// gives a window scan the key and the position.
 struct HitsF32 {
     using T = float4;
-    static constexpr bool kPhiArray = false;
     __device__ __forceinline__ static float round(float v) { return v; }
+    // w: phi16 << 16 | anything
     __device__ __forceinline__ static float4 load(const T* p, int i) { return p[i]; }
-    __device__ __forceinline__ static void store(T* p, int64_t i, float4 c, uint32_t ph)
+    __device__ __forceinline__ static void store(T* p, uint16_t*, int64_t at, float4 c, uint32_t ph, int i)
     {
-        c.w = __int_as_float((int)(ph << 16) | __float_as_int(c.w));
-        p[i] = c;
+        c.w = __int_as_float((int)(ph << 16) | i);
+        p[at] = c;
     }
-    __device__ __forceinline__ static uint32_t key(float4 c, const uint16_t*, int)
-    {
-        return (uint32_t)__float_as_int(c.w);
-    }
-    __device__ __forceinline__ static uint32_t phi_at(const T* p, const uint16_t*, int i)
-    {
-        return (uint32_t)__float_as_int(p[i].w) >> 16;
-    }
+    __device__ __forceinline__ static uint32_t phi(const T* p, int i) { return (uint32_t)__float_as_int(p[i].w) >> 16; }
+    __device__ __forceinline__ static int index(float4 c, const uint16_t*, int) { return __float_as_int(c.w) & 0xFFFF; }
 };
 
 struct HitsF16 {
     using T = ushort4;
-    static constexpr bool kPhiArray = true;
     __device__ __forceinline__ static float round(float v) { return __half2float(__float2half_rn(v)); }
     __device__ __forceinline__ static float4 load(const T* p, int i)
     {
         const ushort4 u = p[i];
         return make_float4(__half2float(__ushort_as_half(u.x)), __half2float(__ushort_as_half(u.y)),
-                           __half2float(__ushort_as_half(u.z)), __int_as_float((int)u.w));
+                           __half2float(__ushort_as_half(u.z)), __int_as_float((int)((uint32_t)u.w << 16)));
     }
-    __device__ __forceinline__ static void store(T* p, int64_t i, float4 c, uint32_t)
+    __device__ __forceinline__ static void store(T* p, uint16_t* idx, int64_t at, float4 c, uint32_t ph, int i)
     {
-        p[i] = make_ushort4(__half_as_ushort(__float2half_rn(c.x)), __half_as_ushort(__float2half_rn(c.y)),
-                            __half_as_ushort(__float2half_rn(c.z)), (unsigned short)__float_as_int(c.w));
+        p[at] = make_ushort4(__half_as_ushort(__float2half_rn(c.x)), __half_as_ushort(__float2half_rn(c.y)),
+                             __half_as_ushort(__float2half_rn(c.z)), (unsigned short)ph);
+        idx[at] = (uint16_t)i;
     }
-    __device__ __forceinline__ static uint32_t key(float4, const uint16_t* ph, int i) { return (uint32_t)ph[i] << 16; }
-    __device__ __forceinline__ static uint32_t phi_at(const T*, const uint16_t* ph, int i) { return ph[i]; }
+    __device__ __forceinline__ static uint32_t phi(const T* p, int i) { return p[i].w; }
+    __device__ __forceinline__ static int index(float4, const uint16_t* idx, int i) { return idx[i]; }
 };
 
-// Event-local input index in a loaded record (below 2^14).
-__device__ __forceinline__ int index_of(float4 c) { return __float_as_int(c.w) & 0xFFFF; }
-
-// Sorted hits of one event: hit p as float4, its phi16.
+// Sorted hits of one event: hit p as float4, its phi16 and its event-local
+// input index (below 2^14).
 template <class HS>
 struct HitArr {
     const typename HS::T* p;
-    const uint16_t* ph;
+    const uint16_t* idx;
     __device__ __forceinline__ float4 operator[](int i) const { return HS::load(p, i); }
-    // record and its phi16 << 16 | low bits
-    __device__ __forceinline__ float4 get(int i, uint32_t& key) const
-    {
-        const float4 c = HS::load(p, i);
-        key = HS::key(c, ph, i);
-        return c;
-    }
-    __device__ __forceinline__ uint32_t phi(int i) const { return HS::phi_at(p, ph, i); }
+    __device__ __forceinline__ uint32_t phi(int i) const { return HS::phi(p, i); }
+    __device__ __forceinline__ int index(float4 c, int i) const { return HS::index(c, idx, i); }
 };
 
 // What one event's search sees: its sorted hits (read-only) and its scratch.
 template <class HS>
 struct Region {
     HitArr<HS> coords;
-    const uint16_t* bucket;     // first sorted position of each (module, phi16 >> 10)
+    const uint16_t* bucket;     // first sorted position of each (module, phi16 >> 9)
     uint32_t* list;
     uint16_t* prev;
     unsigned long long* claim;  // the search's claim of sorted position p is claim[p & cmask]
@@ -281,7 +267,7 @@ __device__ inline Region<HS> region_of(const Sorted& O, int M, int e, int off, c
                                       int64_t r, int cap)
 {
     Region<HS> R;
-    R.coords = HitArr<HS>{(const typename HS::T*)O.coords + off, O.phi + off};
+    R.coords = HitArr<HS>{(const typename HS::T*)O.coords + off, O.index + off};
     R.bucket = O.bucket + (int64_t)e * (M << kBucketBits);
     R.list = W.list + hb;
     R.prev = W.prev + hb;
@@ -338,23 +324,28 @@ __device__ __forceinline__ int bucket_of(int m, uint32_t phi16)
     return (m << kBucketBits) | (int)(phi16 >> (16 - kBucketBits));
 }
 
-constexpr int kShortBucket = 32;    // buckets up to this size are sorted by one thread
+// Hits of buckets up to this size count the smaller keys, above it a warp sorts
+// the bucket (12 M hits in buckets of 64: 550 us counted, 583 sorted; of 128:
+// 634 sorted either way).
+constexpr int kShortBucket = 96;
 
 // Shared memory of the sort kernel: the bucketed entries phi16 << 14 | input
-// index (4 B per hit), phi16 by input order (2 B per hit; later the list of
-// long buckets) and the bucket counters.
-__host__ __device__ inline size_t sort_layout(int nmax, size_t* off_phi, size_t* off_cnt)
+// index (4 B per hit), phi16 by input order (2 B per hit), the bucket counters
+// (16 bits, an event's hits fit) and the list of long buckets: 115 KB for events
+// of 16384 hits, two blocks an SM with 700 B to spare.
+__host__ __device__ inline size_t sort_layout(int nmax, size_t* off_phi, size_t* off_cnt, size_t* off_long)
 {
     size_t o = align16(4 * (size_t)nmax);
     *off_phi = o;  o = align16(o + 2 * (size_t)nmax);
-    *off_cnt = o;  o = align16(o + 4 * (size_t)kSortBuckets);
+    *off_cnt = o;  o = align16(o + 2 * (size_t)kSortBuckets);
+    *off_long = o; o = align16(o + 2 * (size_t)(nmax / kShortBucket + 1));
     return o;
 }
 
 size_t sort_smem_bytes(int nmax)
 {
-    size_t a, b;
-    return sort_layout(nmax, &a, &b);
+    size_t a, b, c;
+    return sort_layout(nmax, &a, &b, &c);
 }
 
 // Ascending sort of a[0, s) by one warp, in place: a bitonic network in the
@@ -397,9 +388,13 @@ __device__ void warp_bitonic(uint32_t* a, int s)
 
 // One block per event: phi16, stable sort by (module, phi16) in shared
 // memory, gather of the sorted hits.  A counting pass puts every hit into its
-// (module, top six bits of phi16) bucket; each bucket is then sorted by
-// phi16 << 14 | input index, a unique key, so the order is the one of a
-// stable sort by (module, phi16).  Status SBT_ERR_ARG for a module id out of
+// (module, top bits of phi16) bucket; within it, a hit's place is the number
+// of smaller keys phi16 << 14 | input index (unique, so the order is the one
+// of a stable sort by (module, phi16)), counted by the hit's own thread: a
+// bucket holds about one hit, and nothing has to be moved once the place is
+// known (moving entries into order bucket by bucket and inverting the order
+// took two more passes: 92 M hits 1280 -> 1190 us).  Long buckets are sorted by
+// a warp each, and their hits look their place up.  Status SBT_ERR_ARG for a module id out of
 // range or a hit range [offsets[e], offsets[e+1]) that is not inside
 // [0, n_hits) (no later kernel reads or writes anything of such an event),
 // SBT_ERR_CAPACITY above the configured hit limit.
@@ -408,11 +403,13 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort(DevConfig C, Inputs in
 {
     constexpr int NT = kSortThreads;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    size_t ophi, ocnt;
-    sort_layout(C.nmax, &ophi, &ocnt);
+    size_t ophi, ocnt, olong;
+    sort_layout(C.nmax, &ophi, &ocnt, &olong);
     uint32_t* ent = (uint32_t*)smem_raw;
     uint16_t* phi = (uint16_t*)(smem_raw + ophi);
-    int* cnt = (int*)(smem_raw + ocnt);
+    uint16_t* cnt = (uint16_t*)(smem_raw + ocnt);
+    uint32_t* cntw = (uint32_t*)cnt;  // two counters a word
+    uint16_t* longb = (uint16_t*)(smem_raw + olong);
     __shared__ int wsum[40];
     __shared__ int err, nlong;
     const int tid = threadIdx.x;
@@ -426,7 +423,8 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort(DevConfig C, Inputs in
         return;
     }
     const int n = (int)n64;
-    for (int b = tid; b < kSortBuckets; b += NT) cnt[b] = 0;
+    const int nb = C.M << kBucketBits;
+    for (int w = tid; w < kSortBuckets / 2; w += NT) cntw[w] = 0u;
     if (tid == 0) {
         err = 0;
         nlong = 0;
@@ -455,7 +453,8 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort(DevConfig C, Inputs in
             }
             const uint32_t ph = phi16_of(HS::round(xs[u]), HS::round(ys[u]));
             phi[i] = (uint16_t)ph;
-            atomicAdd(&cnt[bucket_of(m, ph)], 1);
+            const int b = bucket_of(m, ph);
+            atomicAdd(&cntw[b >> 1], 1u << (16 * (b & 1)));
         }
     }
     __syncthreads();
@@ -463,22 +462,42 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort(DevConfig C, Inputs in
         if (tid == 0) O.status[e] = SBT_ERR_ARG;
         return;
     }
-    // bucket starts: exclusive scan, kSortBuckets / NT consecutive buckets per thread
+    // bucket starts: exclusive scan, kSortBuckets / NT consecutive buckets per
+    // thread; the search's table of starts, and the long buckets
     {
         constexpr int per = kSortBuckets / NT;
-        int v[per];
+        static_assert(per % 8 == 0, "a thread's counters are 16-byte words");
+        uint4* mine = (uint4*)(cnt + tid * per);
         int s = 0;
 #pragma unroll
-        for (int k = 0; k < per; k++) {
-            v[k] = cnt[tid * per + k];
-            s += v[k];
+        for (int k = 0; k < per / 8; k++) {
+            const uint4 v = mine[k];
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int q = 0; q < 4; q++) s += (int)(w[q] & 0xFFFFu) + (int)(w[q] >> 16);
         }
         int total;
         int st = block_exclusive_scan<NT>(s, wsum, &total);
+        uint4* table = (uint4*)(O.bucket + (int64_t)e * nb) + tid * (per / 8);
+        static_assert((1 << kBucketBits) % per == 0, "a module's first bucket is a thread's first");
+        if (tid * per < nb && (tid * per) % (1 << kBucketBits) == 0)
+            O.modoff[(int64_t)e * (C.M + 1) + ((tid * per) >> kBucketBits)] = st;
+        if (tid == 0) O.modoff[(int64_t)e * (C.M + 1) + C.M] = n;
 #pragma unroll
-        for (int k = 0; k < per; k++) {
-            cnt[tid * per + k] = st;
-            st += v[k];
+        for (int k = 0; k < per / 8; k++) {
+            const uint4 v = mine[k];
+            uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const int c0 = (int)(w[q] & 0xFFFFu), c1 = (int)(w[q] >> 16);
+                const int b = tid * per + 8 * k + 2 * q;
+                if (c0 > kShortBucket) longb[atomicAdd(&nlong, 1)] = (uint16_t)b;
+                if (c1 > kShortBucket) longb[atomicAdd(&nlong, 1)] = (uint16_t)(b + 1);
+                w[q] = (uint32_t)st | ((uint32_t)(st + c0) << 16);
+                st += c0 + c1;
+            }
+            mine[k] = make_uint4(w[0], w[1], w[2], w[3]);
+            if (tid * per + 8 * k < nb) table[k] = mine[k];
         }
     }
     __syncthreads();
@@ -486,67 +505,55 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort(DevConfig C, Inputs in
     // cnt[b] is the end of bucket b
     for (int i = tid; i < n; i += NT) {
         const uint32_t ph = phi[i];
-        const int m = in.module[off + i];
-        const int p = atomicAdd(&cnt[bucket_of(m, ph)], 1);
+        const int b = bucket_of(in.module[off + i], ph);
+        const int half = 16 * (b & 1);
+        const int p = (int)(atomicAdd(&cntw[b >> 1], 1u << half) >> half) & 0xFFFF;
         ent[p] = (ph << 14) | (uint32_t)i;
     }
     __syncthreads();
-    // short buckets: insertion sort by one thread; long ones listed for a warp
-    uint16_t* longb = phi;  // phi16 by input order is no longer needed
-    for (int b = tid; b < kSortBuckets; b += NT) {
-        const int lo = b > 0 ? cnt[b - 1] : 0, hi = cnt[b];
-        if (hi - lo > kShortBucket) {
-            longb[atomicAdd(&nlong, 1)] = (uint16_t)b;
-            continue;
+    if (nlong > 0) {
+        for (int q = tid >> 5; q < nlong; q += NT / 32) {
+            const int b = longb[q];
+            const int lo = b > 0 ? cnt[b - 1] : 0;
+            warp_bitonic(ent + lo, cnt[b] - lo);
         }
-        for (int k = lo + 1; k < hi; k++) {
-            const uint32_t v = ent[k];
-            int j = k - 1;
-            while (j >= lo && ent[j] > v) {
-                ent[j + 1] = ent[j];
-                j--;
-            }
-            ent[j + 1] = v;
-        }
+        __syncthreads();
     }
-    __syncthreads();
-    for (int q = tid >> 5; q < nlong; q += NT / 32) {
-        const int b = longb[q];
-        const int lo = b > 0 ? cnt[b - 1] : 0;
-        warp_bitonic(ent + lo, cnt[b] - lo);
-    }
-    for (int m = tid; m <= C.M; m += NT)
-        O.modoff[(int64_t)e * (C.M + 1) + m] = m == 0 ? 0 : (m < C.M ? cnt[(m << kBucketBits) - 1] : n);
-    // bucket starts, two per store (the table has an even length)
-    uint32_t* const tab = (uint32_t*)(O.bucket + (int64_t)e * (C.M << kBucketBits));
-    for (int b = 2 * tid; b < C.M << kBucketBits; b += 2 * NT)
-        tab[b >> 1] = (uint32_t)(b > 0 ? cnt[b - 1] : 0) | ((uint32_t)cnt[b] << 16);
-    __syncthreads();
-    // phi16 by sorted position, and the sorted position of every input hit
-    // (in the space of phi16 by input order, free now)
-    uint16_t* rank = phi;
-    for (int p = tid; p < n; p += NT) {
-        const uint32_t en = ent[p];
-        if (HS::kPhiArray) O.phi[off + p] = (uint16_t)(en >> 14);
-        rank[en & 0x3FFFu] = (uint16_t)p;
-    }
-    __syncthreads();
-    // the hits in input order (coalesced loads), each stored at its sorted
-    // position; two per thread per round
+    // the hits in input order (coalesced loads), each stored at its place; two
+    // per thread per round
     for (int i0 = tid; i0 < n; i0 += 2 * NT) {
         float4 c[2];
-        int q[2];
+        int m[2];
 #pragma unroll
         for (int u = 0; u < 2; u++) {
             const int i = i0 + u * NT;
             if (i < n) {
-                c[u] = make_float4(in.x[off + i], in.y[off + i], in.z[off + i], __int_as_float(i));
-                q[u] = rank[i];
+                m[u] = in.module[off + i];
+                c[u] = make_float4(in.x[off + i], in.y[off + i], in.z[off + i], 0.0f);
             }
         }
 #pragma unroll
-        for (int u = 0; u < 2; u++)
-            if (i0 + u * NT < n) HS::store((typename HS::T*)O.coords, (int64_t)off + q[u], c[u], ent[q[u]] >> 14);
+        for (int u = 0; u < 2; u++) {
+            const int i = i0 + u * NT;
+            if (i >= n) continue;
+            const uint32_t ph = phi[i], own = (ph << 14) | (uint32_t)i;
+            const int b = bucket_of(m[u], ph);
+            int lo = b > 0 ? cnt[b - 1] : 0;
+            const int hi = cnt[b];
+            int q = lo;
+            if (hi - lo <= kShortBucket) {
+                for (int k = lo; k < hi; k++) q += ent[k] < own;
+            } else {
+                for (int end = hi; q < end;) {
+                    const int mid = (q + end) >> 1;
+                    if (ent[mid] < own)
+                        q = mid + 1;
+                    else
+                        end = mid;
+                }
+            }
+            HS::store((typename HS::T*)O.coords, O.index, (int64_t)off + q, c[u], ph, i);
+        }
     }
     if (tid == 0) O.status[e] = SBT_OK;
 }
@@ -656,9 +663,8 @@ __device__ __forceinline__ unsigned long long best_hit(const DevConfig& C, const
             }
             const int end = b;
             do {
-                uint32_t key;
-                const float4 c = R.coords.get(b, key);
-                if (key - lo > width) break;
+                const float4 c = R.coords[b];
+                if ((uint32_t)__float_as_int(c.w) - lo > width) break;
                 const float sc = scatter_of(c, xp, yp);
                 if (sc <= best && sc < cut && (sc < best || b < bb) && G::on(plane, c.x) && !flagged(S, b)) {
                     best = sc;
@@ -1083,7 +1089,7 @@ __device__ void output_stage(int e, int off, const Region<HS>& R, const Smem& S,
         for (int j = nh - 1; j >= 0; j--) {
             const int nq = R.prev[q];
             const float4 c = R.coords[q];
-            const int i = index_of(c);
+            const int i = R.coords.index(c, q);
             hits[u + j] = make_float4(c.x, c.y, c.z, __int_as_float(off + i));
             mn = i < mn ? i : mn;
             q = nq;
@@ -1570,9 +1576,9 @@ __global__ void k_debug_sort_copy(DevConfig C, Inputs in, Sorted O, uint16_t* ph
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < in.n_hits) {
-        const float4 c = HS::load((const typename HS::T*)O.coords, i);
-        phi16[i] = (uint16_t)(HS::key(c, O.phi, i) >> 16);
-        perm[i] = index_of(c);
+        const HitArr<HS> hits{(const typename HS::T*)O.coords, O.index};
+        phi16[i] = (uint16_t)hits.phi((int)i);
+        perm[i] = hits.index(hits[(int)i], (int)i);
     }
     if (i < (int64_t)in.n_events * (C.M + 1)) modoff[i] = O.modoff[i];
 }

@@ -131,6 +131,39 @@ def test_sort_crowded_buckets_bit_exact(sbt):
     assert np.array_equal(mo.cpu().numpy()[0], o)
 
 
+@pytest.mark.parametrize("fp16", [0, 1])
+@pytest.mark.parametrize("size", [1, 2, 95, 96, 97, 128, 129, 300])
+def test_sort_bucket_sizes_bit_exact(sbt, size, fp16):
+    """Buckets at the size up to which hits count the smaller keys and above
+    which a warp sorts them: in the first and last bucket of a module, in
+    neighbouring buckets, with equal phi16 values among them."""
+    rng = np.random.default_rng(size)
+    u = 2 * np.pi / 65536
+    parts = []
+    for module, first in ((0, 0), (0, 127), (5, 64), (5, 65), (51, 127)):
+        q = rng.integers(512 * first + 8, 512 * first + 504, size)
+        q[: size // 3] = q[0]
+        parts.append((q * u, np.full(size, module)))
+    ang = np.concatenate([p[0] for p in parts])
+    m = np.concatenate([p[1] for p in parts]).astype(np.int32)
+    perm0 = rng.permutation(len(m))
+    ang, m = ang[perm0], m[perm0]
+    x, y = (30.0 * np.cos(ang)).astype(np.float32), (30.0 * np.sin(ang)).astype(np.float32)
+    ev = arrays(x, y, MZ[m], m)
+    h = sbt.sbt_create(MZ, sbt.default_config(fp16_hits=fp16, **CFG))
+    try:
+        phi, perm, mo = sbt.sbt_debug_sort(h, *[to_dev(ev)[i] for i in (0, 1, 3, 4)])
+        torch.cuda.synchronize()
+    finally:
+        h.close()
+    if fp16:
+        x, y = (a.astype(np.float16).astype(np.float32) for a in (x, y))
+    p, o, ph = oracle.sort_event(x, y, ev.module, 52)
+    assert np.array_equal(perm.cpu().numpy(), p)
+    assert np.array_equal(phi.cpu().numpy().view(np.uint16), ph)
+    assert np.array_equal(mo.cpu().numpy()[0], o)
+
+
 @pytest.mark.parametrize("batched", [False, True])
 def test_small_workload_bit_exact(sbt, handle, batched):
     ev = synth.make_events(1, workers=1)
