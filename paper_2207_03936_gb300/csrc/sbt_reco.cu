@@ -636,8 +636,10 @@ constexpr unsigned long long kNoHit = ~0ull;
 // bound by the instructions of its longest lane (windows hold 2 to 3 hits on
 // average, the longest of a warp about ten), so the loop tests one key, the
 // scatter and the end; what concerns the few hits under the best scatter so
-// far stands in the branch.
-template <class G, class HS>
+// far stands in the branch.  kAhead: each round loads the next hit too (blocks
+// of 512, which have the registers: one event 212 -> 206 us; at 32 registers
+// it spills).
+template <bool kAhead, class G, class HS>
 __device__ __forceinline__ unsigned long long best_hit(const DevConfig& C, const Smem& S, const Region<HS>& R,
                                                        int t, float3 c0, float3 d0, float cut, float sqrt_cut,
                                                        uint32_t hi)
@@ -662,15 +664,27 @@ __device__ __forceinline__ unsigned long long best_hit(const DevConfig& C, const
                 width = ~0u;
             }
             const int end = b;
+            auto test = [&](float4 c, int p) {
+                const float sc = scatter_of(c, xp, yp);
+                if (sc <= best && sc < cut && (sc < best || p < bb) && G::on(plane, c.x) && !flagged(S, p)) {
+                    best = sc;
+                    bb = p;
+                }
+            };
+            auto outside = [&](float4 c) { return (uint32_t)__float_as_int(c.w) - lo > width; };
             do {
                 const float4 c = R.coords[b];
-                if ((uint32_t)__float_as_int(c.w) - lo > width) break;
-                const float sc = scatter_of(c, xp, yp);
-                if (sc <= best && sc < cut && (sc < best || b < bb) && G::on(plane, c.x) && !flagged(S, b)) {
-                    best = sc;
-                    bb = b;
+                const int next = b + 1 < b1 ? b + 1 : b0;
+                float4 d;
+                if (kAhead) d = R.coords[next];
+                if (outside(c)) break;
+                test(c, b);
+                b = next;
+                if (kAhead) {
+                    if (next == end || outside(d)) break;
+                    test(d, next);
+                    b = next + 1 < b1 ? next + 1 : b0;
                 }
-                b = b + 1 < b1 ? b + 1 : b0;
             } while (b != end);
         }
     }
@@ -703,7 +717,7 @@ __device__ __forceinline__ int lower_bound_hi16(const uint32_t* keys, int n, uin
 constexpr int kSeedLanes = 4;
 constexpr int kSeedGroups = 32 / kSeedLanes;
 
-// Seeding for middle hit c on module s+1 (c < 0: none) by kSeedLanes lanes:
+// Seeding for middle hit c on module s+1 (c < 0: none; phi16 phc) by kSeedLanes lanes:
 // the unflagged hits of module s nearest to c in phi (all hits at the K-th
 // smallest distance included), each extrapolated through c to module s+2,
 // where the unflagged hit of least scatter under the cut is sought; the kept
@@ -712,15 +726,14 @@ constexpr int kSeedGroups = 32 / kSeedLanes;
 // `nu` of them, so the nearest-first walk visits no flagged hit; the lanes
 // walk together and take the candidates in turn.  Every lane of the group
 // returns the triplet as scatter bits << 32 | a << 16 | b, or kNoHit.
-template <class G, class HS>
+template <bool kAhead, class G, class HS>
 __device__ __forceinline__ unsigned long long seed_group(const DevConfig& C, const Smem& S,
-                                                         const Region<HS>& R, int s, int c,
+                                                         const Region<HS>& R, int s, int c, uint32_t phc,
                                                          const uint32_t* outer, int nu, float sqrt_cut)
 {
     unsigned long long best = kNoHit;
     if (c >= 0) {
         const int q = threadIdx.x & (kSeedLanes - 1);
-        const uint32_t phc = R.coords.phi(c);
         int up = lower_bound_hi16(outer, nu, phc);
         int dn = up - 1;
         if (up == nu) up = 0;
@@ -750,7 +763,7 @@ __device__ __forceinline__ unsigned long long seed_group(const DevConfig& C, con
             }
             if (a >= 0) {
                 const float4 Cc = R.coords[c];
-                const unsigned long long v = best_hit<G>(C, S, R, s + 2, make_float3(Cc.x, Cc.y, Cc.z),
+                const unsigned long long v = best_hit<kAhead, G>(C, S, R, s + 2, make_float3(Cc.x, Cc.y, Cc.z),
                                                          sub_rn(Cc, R.coords[a]), C.S_seed, sqrt_cut, (uint32_t)a);
                 best = v < best ? v : best;
             }
@@ -806,7 +819,7 @@ __device__ __forceinline__ FTrack make_track(int h0, int h1, int h2, int key, in
 // Following search of one forming track to module t and its claims: the new
 // hit, and for a 3-hit track also its three hits.  A 3-hit track with a
 // flagged hit cannot extend any more and is marked dead.
-template <class G, class HS>
+template <bool kAhead, class G, class HS>
 __device__ __forceinline__ void follow_and_claim(const DevConfig& C, const Smem& S, const Region<HS>& R,
                                                  int t, unsigned long long tag, float sqrt_cut,
                                                  FTrack& T)
@@ -816,7 +829,7 @@ __device__ __forceinline__ void follow_and_claim(const DevConfig& C, const Smem&
         return;
     }
     const float4 L = R.coords[T.h2];
-    const unsigned long long best = best_hit<G>(C, S, R, t, make_float3(L.x, L.y, L.z), sub_rn(L, R.coords[T.h1]),
+    const unsigned long long best = best_hit<kAhead, G>(C, S, R, t, make_float3(L.x, L.y, L.z), sub_rn(L, R.coords[T.h1]),
                                                 C.S_follow, sqrt_cut, 0u);
     if (best != kNoHit) {
         const int b = (int)(best & 0xFFFFu);
@@ -837,7 +850,9 @@ __device__ __forceinline__ void follow_and_claim(const DevConfig& C, const Smem&
 
 // Iterative seeding and following.  Returns false (uniformly) on overflow.
 // Per module triplet (s, s+1, s+2) three phases separated by barriers:
-//   P0  work lists: unflagged middle hits of s+1, unflagged hits of s in order;
+//   P0  work lists: unflagged middle hits of s+1, unflagged hits of s in order,
+//       both as phi16 << 16 | position; the last warp walks module s alone (it
+//       holds the barrier), the others share module s+1;
 //   P1  seeding, kSeedLanes lanes per middle hit, and following of the forming
 //       tracks to t = s+3 with claims: a warp keeps its new seeds in its lanes
 //       and fills the other lanes with old tracks from a shared counter, so
@@ -855,6 +870,7 @@ __device__ bool search_stage(const DevConfig& C, const Region<HS>& R, const Smem
     int* misc = S.misc;
     const int cap = C.fcap > 0 ? min(C.fcap, forming_capacity(n)) : forming_capacity(n);
     const float sq_seed = sqrtf(C.S_seed), sq_follow = sqrtf(C.S_follow);
+    constexpr bool kAhead = NT == 512;
     uint32_t* list = R.list;
     int cur = 0;
     for (int s = 0; s + 2 <= M - 1; ++s) {
@@ -869,14 +885,14 @@ __device__ bool search_stage(const DevConfig& C, const Region<HS>& R, const Smem
         }
         const int c0 = S.modoff[s + 1], c1 = S.modoff[s + 2];
         uint32_t* outer = list + (c1 - c0);
-        for (int base = c0 + (tid & ~31); base < c1; base += NT) {
+        for (int base = c0 + (tid & ~31); base < c1 && (tid >> 5) < NT / 32 - 1; base += NT - 32) {
             const int c = base + lane;
             const bool ok = c < c1 && !flagged(S, c);
             const unsigned m = __ballot_sync(0xFFFFFFFFu, ok);
             int pos = 0;
             if (lane == 0 && m) pos = atomicAdd(&misc[kList], __popc(m));
             pos = __shfl_sync(0xFFFFFFFFu, pos, 0);
-            if (ok) list[pos + __popc(m & ((1u << lane) - 1u))] = (uint32_t)c;
+            if (ok) list[pos + __popc(m & ((1u << lane) - 1u))] = (R.coords.phi(c) << 16) | (uint32_t)c;
         }
         if ((tid >> 5) == NT / 32 - 1) {
             const int o0 = S.modoff[s], o1 = S.modoff[s + 1];
@@ -904,8 +920,9 @@ __device__ bool search_stage(const DevConfig& C, const Region<HS>& R, const Smem
         for (;;) {
             if (i0 < nl) {
                 const int i = i0 + lane / kSeedLanes;
-                const int c = i < nl ? (int)list[i] : -1;
-                const unsigned long long best = seed_group<G>(C, S, R, s, c, outer, nu, sq_seed);
+                const uint32_t mk = i < nl ? list[i] : 0u;
+                const int c = i < nl ? (int)(mk & 0xFFFFu) : -1;
+                const unsigned long long best = seed_group<kAhead, G>(C, S, R, s, c, mk >> 16, outer, nu, sq_seed);
                 if (best != kNoHit && lane % kSeedLanes == batch) {
                     na = (int)(best >> 16) & 0xFFFF;
                     nc = c;
@@ -939,7 +956,7 @@ __device__ bool search_stage(const DevConfig& C, const Region<HS>& R, const Smem
                 slot = -1;
             }
             if (slot >= 0) {
-                if (follow) follow_and_claim<G>(C, S, R, t, tag, sq_follow, T);
+                if (follow) follow_and_claim<kAhead, G>(C, S, R, t, tag, sq_follow, T);
                 Fc[slot] = T;
             }
             nc = -1;
