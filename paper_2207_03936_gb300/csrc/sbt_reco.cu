@@ -202,10 +202,11 @@ __device__ __forceinline__ void set_flag(const Smem& S, int p) { atomicOr(&S.fla
 // gives a window scan the key and the position.
 struct HitsF32 {
     using T = float4;
+    static constexpr bool kIndexArray = false;
     __device__ __forceinline__ static float round(float v) { return v; }
     // w: phi16 << 16 | anything
     __device__ __forceinline__ static float4 load(const T* p, int i) { return p[i]; }
-    __device__ __forceinline__ static void store(T* p, uint16_t*, int64_t at, float4 c, uint32_t ph, int i)
+    __device__ __forceinline__ static void store(T* p, int64_t at, float4 c, uint32_t ph, int i)
     {
         c.w = __int_as_float((int)(ph << 16) | i);
         p[at] = c;
@@ -216,6 +217,7 @@ struct HitsF32 {
 
 struct HitsF16 {
     using T = ushort4;
+    static constexpr bool kIndexArray = true;
     __device__ __forceinline__ static float round(float v) { return __half2float(__float2half_rn(v)); }
     __device__ __forceinline__ static float4 load(const T* p, int i)
     {
@@ -223,11 +225,10 @@ struct HitsF16 {
         return make_float4(__half2float(__ushort_as_half(u.x)), __half2float(__ushort_as_half(u.y)),
                            __half2float(__ushort_as_half(u.z)), __int_as_float((int)((uint32_t)u.w << 16)));
     }
-    __device__ __forceinline__ static void store(T* p, uint16_t* idx, int64_t at, float4 c, uint32_t ph, int i)
+    __device__ __forceinline__ static void store(T* p, int64_t at, float4 c, uint32_t ph, int)
     {
         p[at] = make_ushort4(__half_as_ushort(__float2half_rn(c.x)), __half_as_ushort(__float2half_rn(c.y)),
                              __half_as_ushort(__float2half_rn(c.z)), (unsigned short)ph);
-        idx[at] = (uint16_t)i;
     }
     __device__ __forceinline__ static uint32_t phi(const T* p, int i) { return p[i].w; }
     __device__ __forceinline__ static int index(float4, const uint16_t* idx, int i) { return idx[i]; }
@@ -552,8 +553,18 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort(DevConfig C, Inputs in
                         end = mid;
                 }
             }
-            HS::store((typename HS::T*)O.coords, O.index, (int64_t)off + q, c[u], ph, i);
+            HS::store((typename HS::T*)O.coords, (int64_t)off + q, c[u], ph, i);
+            if (HS::kIndexArray) phi[i] = (uint16_t)q;  // read by this thread alone
         }
+    }
+    if (HS::kIndexArray) {
+        // the input indices by place, through the space of the entries, so that
+        // they leave coalesced (scattered 2-byte stores: sort of 35 M hits 475 us)
+        uint16_t* idx = (uint16_t*)ent;
+        __syncthreads();
+        for (int i = tid; i < n; i += NT) idx[phi[i]] = (uint16_t)i;
+        __syncthreads();
+        for (int p = tid; p < n; p += NT) O.index[off + p] = idx[p];
     }
     if (tid == 0) O.status[e] = SBT_OK;
 }
