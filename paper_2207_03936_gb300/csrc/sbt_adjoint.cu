@@ -68,7 +68,7 @@ constexpr int kAdjAxes = 5;
 // tracks).
 int adjoint_blocks(int sm_count, int n_tracks)
 {
-    return std::max(1, std::min(kAdjBlocksPerSM * std::max(sm_count, 1), (n_tracks + 31) / 32));
+    return std::max(1, std::min(kAdjBlocksPerSM * std::max(sm_count, 1), n_tracks / 32 + 1));
 }
 
 __device__ __forceinline__ double warp_sum(double v)

@@ -841,7 +841,8 @@ sbt_status sbt_fit_adjoint(sbt_handle* h, const float* x, const float* y, const 
         return fail(h, SBT_ERR_ARG, "NULL argument");
     AdjointWork W;
     W.blocks = adjoint_blocks(h->sm_count, n_tracks);
-    size_t need = sizeof(double) * adjoint_partial_entries(h->C.M, W.blocks);
+    // room for the largest launch at once, so that only the first call allocates
+    size_t need = sizeof(double) * adjoint_partial_entries(h->C.M, adjoint_blocks(h->sm_count, INT32_MAX));
     cudaError_t e = h->misc_arena.reserve(std::max(need, h->misc_arena.bytes));
     if (e != cudaSuccess) return cuda_fail(h, e, "adjoint allocation");
     W.partial = (double*)h->misc_arena.base;
