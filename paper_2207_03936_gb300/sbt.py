@@ -316,9 +316,10 @@ def sbt_fit_adjoint(h: Handle, x, y, z, module, hit_offsets, track_hits, align,
     with_skipped adds the number of tracks without a straight-line fit or
     with an index out of range ([1] int32), which contribute nothing."""
     f32, i32, f64 = torch.float32, torch.int32, torch.float64
-    chi2 = torch.zeros(1, dtype=f64, device=x.device)
-    grad = torch.zeros(h.n_modules * 6, dtype=f64, device=x.device) if want_grad else None
-    skipped = torch.zeros(1, dtype=i32, device=x.device) if with_skipped else None
+    # written whole by the call
+    chi2 = torch.empty(1, dtype=f64, device=x.device)
+    grad = torch.empty(h.n_modules * 6, dtype=f64, device=x.device) if want_grad else None
+    skipped = torch.empty(1, dtype=i32, device=x.device) if with_skipped else None
     st = lib().sbt_fit_adjoint(h.h, _ptr(x, f32, "x"), _ptr(y, f32, "y"), _ptr(z, f32, "z"),
                                _ptr(module, i32, "module"), x.numel(),
                                _ptr(hit_offsets, i32, "hit_offsets"),
