@@ -24,9 +24,9 @@ std::string g_create_error;
 // relative sizes kChunkWeights (small first chunk: short start-up; sizes
 // growing by at most 1.6x; smaller last chunks: short download at the end).
 // From kLargeBatchEvents on, kChunkWeightsLarge: uploads (about 0.5 us per
-// event while downloads share the link) and reconstruction (about 0.47 us
-// per event, plus about 0.7 ms per chunk for the tail of its search and its
-// short kernels) run at nearly the same rate, so after a short ramp the
+// event while downloads share the link) and reconstruction (about 0.41 us
+// per event, 0.47 when the weights were chosen, plus about 0.7 ms per chunk for
+// the tail of its search and its short kernels) run at nearly the same rate, so after a short ramp the
 // chunks stay level at about 11k events and only the last one is small.
 constexpr int64_t kChunkEvents = 12500;
 constexpr int64_t kLargeBatchEvents = 60000;

@@ -4,7 +4,7 @@
 // of the paper).  Two kernels per event:
 //   1. k_sort: phi16 of every hit and its order by (module, phi16, input
 //      index) from one counting pass into (module, coarse phi) buckets and a
-//      sort inside each bucket, in shared memory (section "Sort by phi"); the
+//      count inside each bucket, in shared memory (section "Sort by phi"); the
 //      sorted hits are written as AoS records (x, y, z, phi16 and input
 //      index: float4, or fp16 x, y, z and phi16 with the index beside), with
 //      the start of every bucket;
@@ -151,7 +151,7 @@ enum Misc {
 // Per-block shared memory of the search: flag bits, module offsets, counters,
 // each sized to what the configuration needs.  Everything sized by the event
 // lives in global scratch (L1-resident): shared memory and L1 share one array
-// per SM, so every byte a block holds here comes out of the L1 of 32 resident
+// per SM, so every byte a block holds here comes out of the L1 of the resident
 // events (about n / 8 + 4 M bytes a block).
 struct Smem {
     uint32_t* flag;     // one bit per sorted position
