@@ -274,12 +274,12 @@ def test_block_sizes_agree(sbt, threads):
 
 def test_block_size_follows_the_number_of_events(sbt, handle):
     """The largest and smallest batch of each block size that the library picks
-    by itself (512 threads up to two events an SM, 256 up to eight, then 128),
+    by itself (512 threads up to one event an SM, 256 up to eight, then 128),
     plain and batched."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     ev = synth.make_events(1, 8 * sms + 1, workers=1)
     ref = oracle_of(ev)
-    for e in (1, 2 * sms, 2 * sms + 1, 8 * sms, 8 * sms + 1):
+    for e in (1, sms, sms + 1, 8 * sms, 8 * sms + 1):
         t = int(ref.track_offsets[e])
         hits = int(ref.hit_offsets[t])
         for batched in (False, True):
