@@ -25,10 +25,10 @@
 //           module (a stable counting sort of the tile's hits, integer work);
 //   modules one thread per (module, component): sums into a register that lives
 //           over all tiles.
-// 60 fp64 warp instructions per 32 hits; one warp per track with its lanes over
+// 62 fp64 warp instructions per 32 hits; one warp per track with its lanes over
 // the hits took about 220 (20 of 32 lanes used, shuffled sums, five divisions
-// per track).  2.1 M tracks of 20 hits: 17.5 -> 5.2 ms, the fp64 pipe busy 76%
-// of the time; three hits a thread and tile (smaller tiles) 5.7 ms.
+// per track).  2.1 M tracks of 20 hits: 17.5 -> 5.4 ms, the fp64 pipe busy 77%
+// of the time; three hits a thread and tile (smaller tiles) 11% slower.
 //
 // A track may have any number of hits and several hits on one module (tracks
 // above kTileTrack hits go through a warp each); a track without a
@@ -365,50 +365,71 @@ k_adjoint(DevConfig C, Inputs in, const int32_t* hit_offsets, const int32_t* tra
             const int b = S.first[tr], n = S.first[tr + 1] - b;
             bool bad = false, one = true;
             const double* P = S.tile + b;
-            // sums of four join the sums of all: means and slopes (times 200 mm
-            // of dz) carry the rounding that the residuals feel, and a plain
-            // sum left 20% more of it in the gradient than the shuffled one
-            double sx = 0, sy = 0, sz = 0;
-            for (int j = 0; j < n; j += 4) {
-                double x = 0, y = 0, z = 0;
-#pragma unroll
-                for (int u = 0; u < 4; u++)
-                    if (j + u < n) {
-                        bad |= S.module[b + j + u] == 255;
-                        one &= S.module[b + j + u] == S.module[b];
-                        x += P[0 * kTileHits + j + u];
-                        y += P[1 * kTileHits + j + u];
-                        z += P[2 * kTileHits + j + u];
-                    }
-                sx += x;
-                sy += y;
-                sz += z;
+            // Moments about a point near the mean, their mean part taken out at
+            // the end: the fp32 mean is that point (any point gives the same
+            // line), so the fp64 pipe takes no sums of positions, and the means
+            // carry the rounding of micrometres instead of that of metres.
+            // Gradient error against 128-bit sums, over that of a tree of sums:
+            // 0.92 / 0.94 / 0.98 / 0.99 at 1 / 8 / 60 / 400 events; sums of
+            // positions in fp64, by fours, 1.09 / 1.07 / 1.03 / 1.01 (10000
+            // events 5154 us, here 5363), their means corrected by the sums of
+            // differences 0.92 / 0.93 / 0.98 / 0.99 (5517 us).
+            float sx = 0, sy = 0, sz = 0;
+#pragma unroll 4
+            for (int j = 0; j < n; j++) {
+                bad |= S.module[b + j] == 255;
+                one &= S.module[b + j] == S.module[b];
+                sx += (float)P[0 * kTileHits + j];
+                sy += (float)P[1 * kTileHits + j];
+                sz += (float)P[2 * kTileHits + j];
             }
             if (n > 0 && (bad || one)) {
                 S.skip[tr] = 1;
                 skipped++;
             } else if (n > 0) {
                 Line l;
-                l.xm = sx / n;
-                l.ym = sy / n;
-                l.zm = sz / n;
-                double szz = 0, szx = 0, szy = 0;
+                const float inv = 1.0f / (float)n;
+                const auto near_mean = [&](float sum, const double* v) {
+                    if (isfinite(sum)) return (double)(sum * inv);
+                    double s = 0;  // beyond fp32, or not finite: as it is in fp64
+                    for (int j = 0; j < n; j++) s += v[j];
+                    return s / n;
+                };
+                l.xm = near_mean(sx, P);
+                l.ym = near_mean(sy, P + kTileHits);
+                l.zm = near_mean(sz, P + 2 * kTileHits);
+                double szz = 0, szx = 0, szy = 0, cx = 0, cy = 0, cz = 0;
                 for (int j = 0; j < n; j += 4) {
                     double zz = 0, zx = 0, zy = 0;
 #pragma unroll
                     for (int u = 0; u < 4; u++)
                         if (j + u < n) {
                             const double dz = P[2 * kTileHits + j + u] - l.zm;
+                            const double dx = P[0 * kTileHits + j + u] - l.xm;
+                            const double dy = P[1 * kTileHits + j + u] - l.ym;
                             zz += dz * dz;
-                            zx += dz * (P[0 * kTileHits + j + u] - l.xm);
-                            zy += dz * (P[1 * kTileHits + j + u] - l.ym);
+                            zx += dz * dx;
+                            zy += dz * dy;
+                            cx += dx;
+                            cy += dy;
+                            cz += dz;
                         }
                     szz += zz;
                     szx += zx;
                     szy += zy;
                 }
+                cx /= n;
+                cy /= n;
+                cz /= n;
+                const double szc = cz * n;
+                szz -= szc * cz;
+                szx -= szc * cx;
+                szy -= szc * cy;
                 l.tx = szx / szz;
                 l.ty = szy / szz;
+                l.xm += cx;
+                l.ym += cy;
+                l.zm += cz;
                 S.line[tr] = l;
             }
         }

@@ -158,3 +158,30 @@ def test_adjoint_tiles(setup, n_tracks, lengths):
     assert abs(float(c.item()) - v) <= 1e-12 * v + hits * (delta / SIGMA) ** 2
     assert np.abs(g.cpu().numpy() - go).max() <= 1e-11 * np.abs(go).max() + hits * 2 * delta / SIGMA ** 2 * 42
     assert torch.equal(c, c2) and torch.equal(g, g2)
+
+
+@pytest.mark.parametrize("value", [3e38, np.inf, np.nan], ids=str)
+def test_adjoint_beyond_fp32_sums(setup, value):
+    """Positions whose fp32 sum overflows keep the fp64 result; infinities and
+    NaN reach the same entries as in the oracle."""
+    sbt, h, ev, ho, th, d = setup
+    x = ev.x.copy()
+    t = int(np.argmax(np.diff(ho)))
+    mine = th[ho[t]:ho[t + 1]]
+    if np.isfinite(value):
+        x[mine] = value * np.linspace(0.5, 1.0, len(mine), dtype=np.float32) ** 2
+    else:
+        x[mine[1]] = value
+    align = np.zeros((52, 6))
+    c, g = sbt.sbt_fit_adjoint(h, torch.from_numpy(x).cuda(), d["y"], d["z"], d["m"], d["ho"], d["th"],
+                               torch.from_numpy(align).cuda())
+    with np.errstate(invalid="ignore"):
+        v, go = oracle.align_chi2(x, ev.y, ev.z, ev.module, ho, th, ev.module_z, align, SIGMA)
+    g = g.cpu().numpy()
+    if np.isfinite(value):
+        assert np.isfinite(go).all() and abs(float(c.item()) - v) <= 1e-12 * v
+        # per parameter: n roundings at the scale of its largest entry
+        assert (np.abs(g - go).max(0) <= 1e-12 * np.abs(go).max(0)).all()
+    else:
+        assert np.isnan(v) and np.isnan(float(c.item()))
+        assert np.isnan(go).any() and (np.isnan(g) == np.isnan(go)).all()
