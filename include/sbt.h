@@ -160,8 +160,8 @@ sbt_status sbt_reconstruct(sbt_handle* h, const float* x, const float* y, const 
  * Same result as sbt_reconstruct, produced by one persistent launch whose
  * blocks take events from a device work queue (sizes alternating between the
  * largest and the smallest events not yet taken); the launch
- * sequence is captured once into a CUDA graph per distinct argument set and
- * replayed.  Block size comes from sbt_autotune when it has run.
+ * sequence is captured into a CUDA graph, which calls with the same arguments
+ * replay as long as h keeps its workspaces.  Block size comes from sbt_autotune when it has run.
  */
 sbt_status sbt_reconstruct_batched(sbt_handle* h, const float* x, const float* y, const float* z,
                                    const int32_t* module, const int32_t* event_offsets,
@@ -293,6 +293,11 @@ sbt_status sbt_reconstruct_noalloc(sbt_handle* h, const float* x, const float* y
 /* Number of kernels the last reconstruction call on h enqueued (launch
  * accounting for benchmarks); 0 before any call. */
 int32_t sbt_last_launch_count(const sbt_handle* h);
+
+/* Number of graphs sbt_reconstruct_batched has captured on h: a call with new
+ * arrays, sizes or launch shape captures one, and so does the first call after
+ * another entry point has replaced a workspace of h. */
+int32_t sbt_graph_captures(const sbt_handle* h);
 
 /* ------------------------------------------------------------ serving --- */
 

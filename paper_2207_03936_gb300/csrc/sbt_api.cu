@@ -42,6 +42,7 @@ static_assert(kWeightedChunks <= kMaxChunks && kWeightedChunksLarge <= kMaxChunk
 struct Arena {
     void* base = nullptr;
     size_t bytes = 0;
+    int64_t allocations = 0;     // times base was replaced
     bool defer = false;          // keep outgrown allocations until release()
     std::vector<void*> retired;
     // Grows geometrically: freeing device memory synchronises the device, so
@@ -62,6 +63,7 @@ struct Arena {
         if (base) retired.push_back(base);
         base = p;
         bytes = need;
+        allocations++;
         return cudaSuccess;
     }
     void release()
@@ -137,9 +139,12 @@ size_t carve_staging(void* base, int64_t n_hits, int64_t n_events, Staging* S)
     return c.off + 256;
 }
 
+// What a captured graph depends on: the caller's arrays, sizes, launch shape and
+// the allocations behind the workspaces (any entry point of the handle may
+// replace one by outgrowing it, and a replay would then use freed memory).
 struct GraphKey {
     const void* ptrs[13];
-    int64_t vals[6];
+    int64_t vals[9];
     bool operator==(const GraphKey& o) const
     {
         return std::memcmp(ptrs, o.ptrs, sizeof(ptrs)) == 0 && std::memcmp(vals, o.vals, sizeof(vals)) == 0;
@@ -164,6 +169,7 @@ struct sbt_handle {
     cudaGraphExec_t exec = nullptr;
     GraphKey key{};
     bool have_key = false;
+    int captures = 0;  // graphs captured so far
     int launches_last = 0;
 };
 
@@ -470,9 +476,6 @@ sbt_status sbt_reconstruct_batched(sbt_handle* h, const float* x, const float* y
     Staging S;
     Work W;
     Sorted O;
-    const void* old_stage = h->stage_arena.base;
-    const void* old_pers = h->pers_arena.base;
-    const void* old_sorted = h->sorted_arena.base;
     if ((st = ensure_staging(h, n_hits, n_events, &S)) != SBT_OK) return st;
     if ((st = ensure_persistent(h, blocks, &W)) != SBT_OK) return st;
     if ((st = ensure_sorted(h, n_hits, n_events, &O)) != SBT_OK) return st;
@@ -487,9 +490,10 @@ sbt_status sbt_reconstruct_batched(sbt_handle* h, const float* x, const float* y
     k.vals[3] = out->cap_hits;
     k.vals[4] = threads;
     k.vals[5] = blocks;
-    const bool moved = old_stage != h->stage_arena.base || old_pers != h->pers_arena.base ||
-                       old_sorted != h->sorted_arena.base;
-    if (!h->exec || !h->have_key || moved || !(k == h->key)) {
+    k.vals[6] = h->stage_arena.allocations;
+    k.vals[7] = h->pers_arena.allocations;
+    k.vals[8] = h->sorted_arena.allocations;
+    if (!h->exec || !h->have_key || !(k == h->key)) {
         if (h->exec) {
             cudaGraphExecDestroy(h->exec);
             h->exec = nullptr;
@@ -514,6 +518,7 @@ sbt_status sbt_reconstruct_batched(sbt_handle* h, const float* x, const float* y
         }
         h->key = k;
         h->have_key = true;
+        h->captures++;
     }
     cudaError_t e = cudaGraphLaunch(h->exec, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "graph launch");
@@ -935,5 +940,8 @@ sbt_status sbt_profile_batched(sbt_handle* h, const float* x, const float* y, co
 
 /* Number of kernels the last reconstruction call enqueued (for launch accounting). */
 int32_t sbt_last_launch_count(const sbt_handle* h) { return h ? h->launches_last : 0; }
+
+/* Number of graphs sbt_reconstruct_batched has captured on the handle. */
+int32_t sbt_graph_captures(const sbt_handle* h) { return h ? h->captures : 0; }
 
 }  // extern "C"

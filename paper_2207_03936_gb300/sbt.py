@@ -83,6 +83,7 @@ def lib() -> ctypes.CDLL:
             "sbt_debug_sort": (_I32, [_P, _P, _P, _P, _P, _I32, _I32, _P, _P, _P, _P]),
             "sbt_debug_phi16": (_I32, [_P, _P, _I32, _P, _P]),
             "sbt_last_launch_count": (_I32, [_P]),
+            "sbt_graph_captures": (_I32, [_P]),
             "sbt_profile_batched": (_I32, [_P, _P, _P, _P, _P, _P, _I32, _I32, _P, _I32, _P, _P]),
         }
         for name, (res, args) in sig.items():
@@ -215,6 +216,9 @@ class Handle:
 
     def last_launch_count(self) -> int:
         return int(lib().sbt_last_launch_count(self.h))
+
+    def graph_captures(self) -> int:
+        return int(lib().sbt_graph_captures(self.h))
 
 
 def sbt_create(module_z, config: Config | None = None, **kw) -> Handle:

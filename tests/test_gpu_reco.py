@@ -516,6 +516,38 @@ def test_last_kernel_of_small_batches(sbt, handle, events):
         assert np.array_equal(chi[:tw].view(np.uint32), ref.chi2[:tw].view(np.uint32)) and (chi[tw:] == -7).all()
 
 
+@pytest.mark.parametrize("other", ["plain", "host", "debug_sort", "autotune", "profile"])
+def test_batched_graph_is_captured_again_after_a_workspace_moved(sbt, other):
+    """A batched call repeated on the same arrays replays its graph; after a
+    larger call through another entry point, which outgrows workspaces of the
+    handle, it captures anew instead of replaying freed addresses."""
+    small, big = synth.make_events(2, 20, workers=1), synth.make_events(2, 1400, workers=1)
+    ref = oracle_of(small)
+    h = sbt.sbt_create(MZ, sbt.default_config(**CFG))
+    try:
+        dev = to_dev(small)
+        out = sbt.TrackOutput.allocate(small.n_events, small.n_hits)
+        for _ in range(2):
+            assert_same(sbt.sbt_reconstruct_batched(h, *dev, out=out).compact(), ref)
+        assert h.graph_captures() == 1
+        args = to_dev(big)
+        if other == "plain":
+            sbt.sbt_reconstruct(h, *args)
+        elif other == "host":
+            sbt.sbt_reconstruct_host(h, *[a.cpu() for a in args])
+        elif other == "debug_sort":
+            sbt.sbt_debug_sort(h, *[args[i] for i in (0, 1, 3, 4)])
+        elif other == "autotune":
+            sbt.sbt_autotune(h, *args)
+        else:
+            sbt.sbt_profile_batched(h, *args, sbt.TrackOutput.allocate(big.n_events, big.n_hits), reps=1)
+        for _ in range(2):
+            assert_same(sbt.sbt_reconstruct_batched(h, *dev, out=out).compact(), ref)
+        assert h.graph_captures() == 2
+    finally:
+        h.close()
+
+
 def test_repeat_runs_are_identical(sbt, handle):
     ev = synth.make_events(2, 200, workers=1)
     a = run_gpu(sbt, handle, ev, True)
