@@ -107,13 +107,14 @@ size_t carve_work(void* base, int64_t hits, int64_t regions, Work* W)
 }
 
 // Sorted hits of a batch (see Sorted).
-size_t carve_sorted(void* base, int64_t n_hits, int64_t n_events, int M, Sorted* O)
+size_t carve_sorted(void* base, int64_t n_hits, int64_t n_events, int M, const Tables& t, Sorted* O)
 {
     Carver c(base);
     Sorted o;
     o.coords = c.take<float4>(n_hits);
     o.index = c.take<uint16_t>(n_hits);
-    o.bucket = c.take<uint16_t>(n_events * (M << kBucketBits));
+    o.bucket = c.take<uint16_t>(table_entries(t, n_hits, n_events));
+    o.tables = t;
     o.modoff = c.take<int32_t>(n_events * (M + 1));
     o.status = c.take<int32_t>(n_events);
     if (O) *O = o;
@@ -161,6 +162,7 @@ struct sbt_handle {
     std::string err;
     Arena plain_arena, pers_arena, stage_arena, host_arena, misc_arena, sorted_arena;
     int concurrent = 1;     // calls of other handles that share the GPU with this one's, itself included
+    bool serving = false;   // of a serving slot
     int tuned_threads = 0;
     int tuned_blocks_per_sm = 0;  // resident blocks per SM of the persistent launch (0: occupancy limit)
     cudaStream_t cap_stream = nullptr;
@@ -249,10 +251,11 @@ Inputs make_inputs(const float* x, const float* y, const float* z, const int32_t
 
 sbt_status ensure_sorted(sbt_handle* h, int64_t n_hits, int64_t n_events, Sorted* O)
 {
-    size_t need = carve_sorted(nullptr, n_hits, n_events, h->C.M, nullptr);
+    const Tables t = handle_tables(h, n_events);
+    size_t need = carve_sorted(nullptr, n_hits, n_events, h->C.M, t, nullptr);
     cudaError_t e = h->sorted_arena.reserve(need);
     if (e != cudaSuccess) return cuda_fail(h, e, "sorted-hit allocation");
-    carve_sorted(h->sorted_arena.base, n_hits, n_events, h->C.M, O);
+    carve_sorted(h->sorted_arena.base, n_hits, n_events, h->C.M, t, O);
     return SBT_OK;
 }
 
@@ -310,9 +313,19 @@ const DevConfig& handle_device_config(const sbt_handle* h) { return h->C; }
 
 int handle_plain_threads(const sbt_handle* h, int64_t n_events) { return default_threads(h, false, n_events); }
 
+Tables handle_tables(const sbt_handle* h, int64_t n_events)
+{
+    const bool full = n_events <= 8 * (int64_t)h->sm_count && !h->serving;
+    return full ? tables_full(h->C.M) : tables_by_hits(h->C.M);
+}
+
 int handle_configured_threads(const sbt_handle* h) { return h->cfg.threads_per_block; }
 
-void handle_set_concurrent(sbt_handle* h, int handles) { h->concurrent = handles; }
+void handle_set_serving(sbt_handle* h, int slots)
+{
+    h->concurrent = slots;
+    h->serving = true;
+}
 
 void handle_set_error(sbt_handle* h, const std::string& msg) { h->err = msg; }
 
@@ -631,7 +644,7 @@ sbt_status sbt_reconstruct_host(sbt_handle* h, const float* x, const float* y, c
     auto chunk_views = [&](int c, Sorted& Oc, Staging& Sc) {
         const int64_t ev0 = e0[c];
         Oc = O;
-        Oc.bucket = O.bucket + ev0 * (h->C.M << kBucketBits);
+        Oc.bucket = O.bucket + ev0 * O.tables.per_event;
         Oc.modoff = O.modoff + ev0 * (h->C.M + 1);
         Oc.status = O.status + ev0;
         Sc = S;

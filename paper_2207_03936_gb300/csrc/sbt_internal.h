@@ -10,11 +10,46 @@
 namespace sbt {
 
 constexpr int kMaxModules = 64;
-// The sort's buckets, top bits of phi16 within a module: about one hit each, so
-// that a window's scan starts near its edge (search of 92 M hits 5.28 ms with 6
-// bits, 5.07 with 7).
-constexpr int kBucketBits = 7;
 constexpr int kMaxHitsPerEvent = 16384;  // the per-event sort runs in shared memory
+// The sort's buckets: a module's hits by the top bits of phi16, at most this
+// many, so that a bucket holds about one hit and a window's scan starts near its
+// edge (search of 92 M hits 5.28 ms with 6 bits, 5.07 with 7).
+constexpr int kBucketBits = 7;
+
+// How a batch's events are bucketed, and where event e, whose hits begin at off,
+// has its table of bucket starts: from per_hit * off + per_event * e on (off
+// rounded down to even, so that tables are whole 16-byte words).  Two forms:
+//   by hits   one to four buckets a hit (7 bits from 2048 hits on 52 modules on),
+//             at least two a module, so that the sort's work and the tables
+//             follow the hits.  With 7 bits for every event the tables were
+//             13 KB an event, 2.7 GB for 200000 events of 20 hits (now 80 MB),
+//             and their sort took 2587 us (now 2201; 5000 events of 686 hits 91
+//             and 86);
+//   full      7 bits for every event, while every event has a block on the GPU
+//             at once (eight blocks of 256 threads an SM): such a call waits for
+//             the longest scans, which begin up to a bucket before their
+//             windows.  16 events of 700 hits: 166 us a call by hits, 151 full.
+struct Tables {
+    int least_bits, per_hit, per_event;
+};
+
+constexpr Tables tables_by_hits(int n_modules) { return {1, 4, ((2 * n_modules + 7) & ~7) + 8}; }
+constexpr Tables tables_full(int n_modules) { return {kBucketBits, 0, n_modules << kBucketBits}; }
+
+constexpr int64_t table_entries(const Tables& t, int64_t n_hits, int64_t n_events)
+{
+    return t.per_hit * n_hits + t.per_event * n_events;
+}
+
+__device__ __forceinline__ int64_t table_base(const Tables& t, int64_t off, int64_t e)
+{
+    return t.per_hit * (off & ~(int64_t)1) + t.per_event * e;
+}
+
+__device__ __forceinline__ int bucket_bits(const Tables& t, int n_hits, int n_modules)
+{
+    return min(kBucketBits, max(t.least_bits, __clz(n_modules) - __clz(n_hits) + 1));
+}
 
 // Method constants and per-event capacities, passed to kernels by value.
 struct DevConfig {
@@ -61,8 +96,9 @@ struct Sorted {
     float4* coords;   // (x, y, z, phi16 << 16 | event-local input index) by sorted position, or
                       // fp16 records
     uint16_t* index;  // event-local input index by sorted position (fp16 records only)
-    uint16_t* bucket; // [n_events * (n_modules << kBucketBits)] event-local start of every
-                      // (module, phi16 >> 9): where a window's scan begins
+    uint16_t* bucket; // [table_entries] event e's from table_base on: event-local start of every
+                      // (module, top bucket_bits bits of phi16), where a window's scan begins
+    Tables tables;
     int32_t* modoff;  // [n_events * (n_modules + 1)] event-local module offsets
     int32_t* status;  // [n_events] SBT_OK, SBT_ERR_ARG or SBT_ERR_CAPACITY after the sort
 };
@@ -156,9 +192,11 @@ size_t adjoint_partial_entries(int M, int blocks);
 const DevConfig& handle_device_config(const sbt_handle* h);
 int handle_plain_threads(const sbt_handle* h, int64_t n_events);
 int handle_configured_threads(const sbt_handle* h);
-// How many handles launch at the same time (the serving slots): their events
-// share the GPU, which decides the block size.
-void handle_set_concurrent(sbt_handle* h, int handles);
+Tables handle_tables(const sbt_handle* h, int64_t n_events);
+// A handle of one of `slots` serving slots: their events share the GPU, which
+// decides the block size, and their tables are sized by the hits, as admission
+// counts them.
+void handle_set_serving(sbt_handle* h, int slots);
 void handle_set_error(sbt_handle* h, const std::string& msg);
 void handle_set_launches(sbt_handle* h, int launches);
 // Workspaces the handle outgrows are kept until sbt_destroy instead of freed

@@ -33,6 +33,9 @@ struct Layout {
     size_t hits, tkey, tinfo, rinfo, tfit, ntracks, nhits, track_base, hit_base, order, queue, total;
 };
 
+// Tables by hits of the largest batch; full ones are used where they fit.
+constexpr int64_t kTableEntries = table_entries(tables_by_hits(kMaxModules), kNoAllocMaxHits, kNoAllocMaxEvents);
+
 constexpr Layout make_layout()
 {
     Layout L{};
@@ -41,7 +44,7 @@ constexpr Layout make_layout()
     size_t o = 0;
     L.coords = o;     o = align256(o + 16 * (size_t)H);
     L.index = o;       o = align256(o + 2 * (size_t)H);
-    L.bucket = o;     o = align256(o + 2 * (size_t)E * (kMaxModules << kBucketBits));
+    L.bucket = o;     o = align256(o + 2 * (size_t)kTableEntries);
     L.modoff = o;     o = align256(o + 4 * (size_t)E * (kMaxModules + 1));
     L.status = o;     o = align256(o + 4 * (size_t)E);
     L.list = o;       o = align256(o + 4 * (size_t)H);
@@ -67,8 +70,9 @@ constexpr Layout make_layout()
 }
 
 constexpr Layout kLayout = make_layout();
+static_assert(kLayout.total < (size_t)56 << 20, "held on every GPU that loads the library");
 
-// The workspace (about 115 MB).  In host code this name is only a host-side
+// The workspace (about 54 MB).  In host code this name is only a host-side
 // stand-in: its device address comes from cudaGetSymbolAddress below.
 __device__ __align__(256) unsigned char g_noalloc_workspace[kLayout.total];
 
@@ -137,6 +141,9 @@ extern "C" sbt_status sbt_reconstruct_noalloc(sbt_handle* h, const float* x, con
     O.coords = (float4*)(base + L.coords);
     O.index = (uint16_t*)(base + L.index);
     O.bucket = (uint16_t*)(base + L.bucket);
+    O.tables = handle_tables(h, n_events);
+    if (table_entries(O.tables, n_hits, n_events) > kTableEntries)
+        O.tables = tables_by_hits(handle_device_config(h).M);
     O.modoff = (int32_t*)(base + L.modoff);
     O.status = (int32_t*)(base + L.status);
     Work W;

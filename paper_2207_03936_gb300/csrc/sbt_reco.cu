@@ -145,7 +145,7 @@ __device__ __forceinline__ void fit_line(int n, Get get, float sigma, float* par
 
 enum Misc {
     kErr = 0, kNFin = 1, kNTl = 2, kEvent = 3, kCMask = 4, kCnt0 = 5, kCnt1 = 6, kWork = 7, kNew = 8, kList = 9,
-    kNOuter = 10, kMiscN = 12
+    kNOuter = 10, kShift = 11, kMiscN = 12
 };
 
 // Per-block shared memory of the search: flag bits, module offsets, counters,
@@ -249,7 +249,7 @@ struct HitArr {
 template <class HS>
 struct Region {
     HitArr<HS> coords;
-    const uint16_t* bucket;     // first sorted position of each (module, phi16 >> 9)
+    const uint16_t* bucket;     // first sorted position of each (module, phi16 >> misc[kShift])
     uint32_t* list;
     uint16_t* prev;
     unsigned long long* claim;  // the search's claim of sorted position p is claim[p & cmask]
@@ -269,7 +269,7 @@ __device__ inline Region<HS> region_of(const Sorted& O, int M, int e, int off, c
 {
     Region<HS> R;
     R.coords = HitArr<HS>{(const typename HS::T*)O.coords + off, O.index + off};
-    R.bucket = O.bucket + (int64_t)e * (M << kBucketBits);
+    R.bucket = O.bucket + table_base(O.tables, off, e);
     R.list = W.list + hb;
     R.prev = W.prev + hb;
     R.claim_all = W.claim + hb;
@@ -319,10 +319,12 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* wsum, int* total
 // ------------------------------------------------------------- sorting ---
 
 constexpr int kSortThreads = 1024;
-constexpr int kSortBuckets = kMaxModules << kBucketBits;  // (module, top bits of phi16)
-__device__ __forceinline__ int bucket_of(int m, uint32_t phi16)
+constexpr int kSortBuckets = kMaxModules << kBucketBits;
+
+// Bucket of a hit on module m: module and the top 16 - shift bits of phi16.
+__device__ __forceinline__ int bucket_of(int m, uint32_t phi16, int shift)
 {
-    return (m << kBucketBits) | (int)(phi16 >> (16 - kBucketBits));
+    return (int)(((uint32_t)m << 16 | phi16) >> shift);
 }
 
 // Hits of buckets up to this size count the smaller keys, above it a warp sorts
@@ -424,8 +426,9 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort(DevConfig C, Inputs in
         return;
     }
     const int n = (int)n64;
-    const int nb = C.M << kBucketBits;
-    for (int w = tid; w < kSortBuckets / 2; w += NT) cntw[w] = 0u;
+    const int shift = 16 - bucket_bits(O.tables, n, C.M);
+    const int nb = C.M << (16 - shift);
+    for (int w = tid; w < (nb + 7) / 8; w += NT) ((uint4*)cnt)[w] = make_uint4(0u, 0u, 0u, 0u);
     if (tid == 0) {
         err = 0;
         nlong = 0;
@@ -454,7 +457,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort(DevConfig C, Inputs in
             }
             const uint32_t ph = phi16_of(HS::round(xs[u]), HS::round(ys[u]));
             phi[i] = (uint16_t)ph;
-            const int b = bucket_of(m, ph);
+            const int b = bucket_of(m, ph, shift);
             atomicAdd(&cntw[b >> 1], 1u << (16 * (b & 1)));
         }
     }
@@ -463,42 +466,34 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort(DevConfig C, Inputs in
         if (tid == 0) O.status[e] = SBT_ERR_ARG;
         return;
     }
-    // bucket starts: exclusive scan, kSortBuckets / NT consecutive buckets per
-    // thread; the search's table of starts, and the long buckets
+    // bucket starts: exclusive scan, eight consecutive buckets per thread; the
+    // search's table of starts, and the long buckets
     {
-        constexpr int per = kSortBuckets / NT;
-        static_assert(per % 8 == 0, "a thread's counters are 16-byte words");
-        uint4* mine = (uint4*)(cnt + tid * per);
+        static_assert(kSortBuckets <= 8 * NT, "one 16-byte word of counters a thread");
+        uint4* mine = (uint4*)cnt + tid;
+        const bool any = 8 * tid < nb;
+        uint32_t w[4] = {0u, 0u, 0u, 0u};
+        if (any) {
+            const uint4 v = *mine;
+            w[0] = v.x, w[1] = v.y, w[2] = v.z, w[3] = v.w;
+        }
         int s = 0;
 #pragma unroll
-        for (int k = 0; k < per / 8; k++) {
-            const uint4 v = mine[k];
-            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int q = 0; q < 4; q++) s += (int)(w[q] & 0xFFFFu) + (int)(w[q] >> 16);
-        }
+        for (int q = 0; q < 4; q++) s += (int)(w[q] & 0xFFFFu) + (int)(w[q] >> 16);
         int total;
         int st = block_exclusive_scan<NT>(s, wsum, &total);
-        uint4* table = (uint4*)(O.bucket + (int64_t)e * nb) + tid * (per / 8);
-        static_assert((1 << kBucketBits) % per == 0, "a module's first bucket is a thread's first");
-        if (tid * per < nb && (tid * per) % (1 << kBucketBits) == 0)
-            O.modoff[(int64_t)e * (C.M + 1) + ((tid * per) >> kBucketBits)] = st;
-        if (tid == 0) O.modoff[(int64_t)e * (C.M + 1) + C.M] = n;
-#pragma unroll
-        for (int k = 0; k < per / 8; k++) {
-            const uint4 v = mine[k];
-            uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        if (any) {
 #pragma unroll
             for (int q = 0; q < 4; q++) {
                 const int c0 = (int)(w[q] & 0xFFFFu), c1 = (int)(w[q] >> 16);
-                const int b = tid * per + 8 * k + 2 * q;
+                const int b = 8 * tid + 2 * q;
                 if (c0 > kShortBucket) longb[atomicAdd(&nlong, 1)] = (uint16_t)b;
                 if (c1 > kShortBucket) longb[atomicAdd(&nlong, 1)] = (uint16_t)(b + 1);
                 w[q] = (uint32_t)st | ((uint32_t)(st + c0) << 16);
                 st += c0 + c1;
             }
-            mine[k] = make_uint4(w[0], w[1], w[2], w[3]);
-            if (tid * per + 8 * k < nb) table[k] = mine[k];
+            *mine = make_uint4(w[0], w[1], w[2], w[3]);
+            ((uint4*)(O.bucket + table_base(O.tables, off, e)))[tid] = *mine;
         }
     }
     __syncthreads();
@@ -506,12 +501,13 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort(DevConfig C, Inputs in
     // cnt[b] is the end of bucket b
     for (int i = tid; i < n; i += NT) {
         const uint32_t ph = phi[i];
-        const int b = bucket_of(in.module[off + i], ph);
+        const int b = bucket_of(in.module[off + i], ph, shift);
         const int half = 16 * (b & 1);
         const int p = (int)(atomicAdd(&cntw[b >> 1], 1u << half) >> half) & 0xFFFF;
         ent[p] = (ph << 14) | (uint32_t)i;
     }
     __syncthreads();
+    if (tid <= C.M) O.modoff[(int64_t)e * (C.M + 1) + tid] = tid > 0 ? cnt[(tid << (16 - shift)) - 1] : 0;
     if (nlong > 0) {
         for (int q = tid >> 5; q < nlong; q += NT / 32) {
             const int b = longb[q];
@@ -538,7 +534,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort(DevConfig C, Inputs in
             const int i = i0 + u * NT;
             if (i >= n) continue;
             const uint32_t ph = phi[i], own = (ph << 14) | (uint32_t)i;
-            const int b = bucket_of(m[u], ph);
+            const int b = bucket_of(m[u], ph, shift);
             int lo = b > 0 ? cnt[b - 1] : 0;
             const int hi = cnt[b];
             int q = lo;
@@ -666,11 +662,14 @@ __device__ __forceinline__ unsigned long long best_hit(const DevConfig& C, const
             int b = b0;
             // keys compared as phi16 << 16 | low bits; without a window every hit is inside
             if (window_of(xp, yp, cut, sqrt_cut, lo, width)) {
-                constexpr uint32_t kIn = (1u << (16 - kBucketBits)) - 1u;
-                b = R.bucket[bucket_of(t, lo)];
+                const int shift = S.misc[kShift];
+                const uint32_t k = (uint32_t)bucket_of(t, lo, shift);
+                b = R.bucket[k];
+                b = max(b, b0);
                 b = b < b1 ? b : b0;
-                width = ((width + (lo & kIn)) << 16) | 0xFFFFu;
-                lo = (lo & ~kIn) << 16;
+                const uint32_t edge = k << shift << 16;  // the bucket's, above the low bits
+                width = ((width + lo) << 16 | 0xFFFFu) - edge;
+                lo = edge;
             } else {
                 width = ~0u;
             }
@@ -1172,7 +1171,8 @@ __device__ void run_event(const DevConfig& C, const Inputs& in, const Sorted& O,
         w = __reduce_max_sync(0xFFFFFFFFu, w);
         const int p2 = w > 1 ? 1 << (32 - __clz(w - 1)) : 1;
         if (tid == 0) S.misc[kCMask] = p2 <= cap ? p2 - 1 : -1;
-        if (tid < kMiscN && tid != kCMask && tid != kEvent) S.misc[tid] = 0;
+        if (tid == 0) S.misc[kShift] = 16 - bucket_bits(O.tables, n, C.M);
+        if (tid < kMiscN && tid != kCMask && tid != kEvent && tid != kShift) S.misc[tid] = 0;
     }
     __syncthreads();
     // the ring starts empty; older claims lose against newer ones by their tag

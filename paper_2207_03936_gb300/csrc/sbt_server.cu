@@ -190,14 +190,14 @@ struct Slot {
     HostBuf<int32_t> hm, hoff;
 };
 
-// Device bytes one batch needs (inputs, outputs and the plain workspace):
-// per hit 16 B inputs, 18 B sorted hits, about 45 B search scratch (claims,
-// links, lists, tracklets, forming and final tracks), about 12 B staging and
-// about 13 B outputs, rounded up; per event its module offsets, counts and
-// bucket table.
-int64_t batch_bytes(int64_t hits, int64_t events)
+// Device bytes one batch needs (inputs, outputs and the plain workspace): per
+// hit 16 B inputs, 26 B sorted hits and window table, 30 B search scratch
+// (lists, links, claims, forming tracks, tracklets, final tracks), 23 B staging
+// and 13 B outputs, rounded up; per event its module offsets, counts and the
+// least window table.
+int64_t batch_bytes(int64_t hits, int64_t events, int n_modules)
 {
-    return hits * 112 + events * (320 + 2 * (sbt::kMaxModules << sbt::kBucketBits)) + (1 << 16);
+    return hits * 112 + events * (320 + 2 * sbt::tables_by_hits(n_modules).per_event) + (1 << 16);
 }
 
 }  // namespace
@@ -320,6 +320,7 @@ bool launch_batch(Slot& sl)
 void launcher_loop(sbt_server* S)
 {
     cudaSetDevice(S->device);
+    const int n_modules = sbt::handle_device_config(S->slots[0]->h).M;
     for (;;) {
         Slot* free_slot = nullptr;
         for (auto& up : S->slots)
@@ -336,7 +337,7 @@ void launcher_loop(sbt_server* S)
                 int64_t hits = 0;
                 while (!S->pending.empty() && (int32_t)take.size() < S->max_batch) {
                     const Request& r = S->pending.front();
-                    const int64_t b = batch_bytes(hits + (int64_t)r.n, (int64_t)take.size() + 1);
+                    const int64_t b = batch_bytes(hits + (int64_t)r.n, (int64_t)take.size() + 1, n_modules);
                     if (S->in_flight_bytes + b > S->budget && (!take.empty() || S->in_flight_bytes > 0))
                         break;
                     hits += (int64_t)r.n;
@@ -518,7 +519,7 @@ sbt_status sbt_server_create(sbt_handle* h, int64_t memory_budget_bytes, int32_t
     }
     for (auto& sl : S->slots) {
         sbt::handle_defer_frees(sl->h);
-        sbt::handle_set_concurrent(sl->h, max_streams);
+        sbt::handle_set_serving(sl->h, max_streams);
     }
     S->allocs0 = g_allocs.load();
     S->launcher = std::thread(launcher_loop, S);

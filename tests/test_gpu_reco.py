@@ -762,6 +762,70 @@ def test_candidate_lanes_and_bucket_windows_bit_exact(sbt, k, per_module):
         h.close()
 
 
+@pytest.mark.parametrize("fp16", [0, 1])
+@pytest.mark.parametrize("tables", ["full", "by hits"])
+def test_window_tables_of_uneven_events_bit_exact(sbt, tables, fp16):
+    """Events on both sides of every size at which the sort's buckets and the
+    window table gain a bit (powers of two: 8 hits to 256 on seven modules),
+    empty ones and odd hit counts among them, on hits without tracks and with
+    wide cuts; in a small batch, where every event has all bits, and in one of
+    more than eight events an SM, where the bits follow the hits."""
+    rng = np.random.default_rng(8)
+    M = 7
+    sizes = [n for k in range(2, 10) for n in (2 ** k - 1, 2 ** k, 2 ** k + 1)] + [0, 1, 0, 700]
+    if tables == "by hits":
+        sizes *= 8 * torch.cuda.get_device_properties(0).multi_processor_count // len(sizes) + 1
+    off = np.concatenate([[0], np.cumsum(rng.permutation(sizes))]).astype(np.int32)
+    n = int(off[-1])
+    ang, r = np.pi + rng.normal(0.0, 1.0, n), rng.uniform(5.1, 9.0, n)
+    module = rng.integers(0, M, n).astype(np.int32)
+    ev = synth.Events((r * np.cos(ang)).astype(np.float32), (r * np.sin(ang)).astype(np.float32), MZ[module],
+                      module, off, np.full(n, -1, np.int32), 0, MZ[:M].copy())
+    # this cut keeps the largest events' forming tracks under n / 12 + 64
+    cfg = dict(CFG, max_scatter_seed=0.02, max_scatter_follow=0.2, max_chi2_tracklet=5000.0)
+    ref = oracle.reconstruct(ev.x, ev.y, ev.z, ev.module, ev.event_offsets, ev.module_z, oracle.config(**cfg),
+                             fp16_hits=bool(fp16))
+    assert ref.n_tracks > 50
+    h = sbt.sbt_create(ev.module_z, sbt.default_config(fp16_hits=fp16, **cfg))
+    try:
+        for batched in (False, True):
+            assert_same(run_gpu(sbt, h, ev, batched), ref)
+        out = sbt.TrackOutput.allocate(ev.n_events, ev.n_hits)
+        assert_same(sbt.sbt_reconstruct_noalloc(h, *to_dev(ev), out=out).compact(), ref)
+        phi, perm, mo = sbt.sbt_debug_sort(h, *[to_dev(ev)[i] for i in (0, 1, 3, 4)])
+        torch.cuda.synchronize()
+    finally:
+        h.close()
+    x, y = (oracle.round_fp16(a) if fp16 else a for a in (ev.x, ev.y))
+    perm, phi, mo = perm.cpu().numpy(), phi.cpu().numpy().view(np.uint16), mo.cpu().numpy()
+    for e in range(ev.n_events):
+        lo, hi = off[e], off[e + 1]
+        p, o, ph = oracle.sort_event(x[lo:hi], y[lo:hi], module[lo:hi], M)
+        assert np.array_equal(perm[lo:hi], p) and np.array_equal(phi[lo:hi], ph) and np.array_equal(mo[e], o)
+
+
+def test_workspace_follows_the_hits_of_tiny_events(sbt):
+    """The sorted-hit workspace of 100000 events of 20 hits stays near what
+    their hits and module offsets take (26 bytes a hit, 450 an event): 97 MB,
+    half as much again where it grows."""
+    E, n = 100000, 20
+    h = sbt.sbt_create(MZ, sbt.default_config(**CFG))
+    try:
+        x = torch.rand(E * n, device="cuda") + 5.1
+        m = torch.arange(E * n, device="cuda", dtype=torch.int32) % 52
+        off = torch.arange(E + 1, device="cuda", dtype=torch.int32) * n
+        sbt.sbt_debug_sort(h, x[:n], x[:n], m[:n], off[:2])
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        free = torch.cuda.mem_get_info()[0]
+        sbt.sbt_debug_sort(h, x, x, m, off)
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        assert free - torch.cuda.mem_get_info()[0] < 160e6
+    finally:
+        h.close()
+
+
 def test_event_ranges_outside_the_hits_are_reported(sbt, handle):
     # events whose hit range ends past n_hits get SBT_ERR_ARG on the device
     # and no tracks; the others are reconstructed as usual.  The hit arrays

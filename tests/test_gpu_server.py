@@ -50,6 +50,24 @@ def test_served_results_equal_results_alone():
         assert r.latency_s > 0
 
 
+def test_admission_counts_the_hits_of_quiet_events():
+    """The bytes a batch counts against the budget follow its hits (112 a hit and
+    600 an event at 52 modules), also for events of a few hundred hits."""
+    from paper_2207_03936_gb300 import sbt
+    ev = synth.make_events(1, 64, workers=1)
+    h = sbt.sbt_create(ev.module_z, sbt.default_config())
+    srv = sbt.Server(h, memory_budget_bytes=256 << 20, max_streams=1, max_batch_events=64)
+    try:
+        srv.submit_schedule(ev, np.zeros(ev.n_events))
+        got = collect(srv, ev.n_events)
+        st = srv.stats()
+    finally:
+        srv.close()
+        h.close()
+    assert len(got) == ev.n_events and all(r.status == 0 for r in got.values())
+    assert 0 < st["peak_bytes"] <= 112 * ev.n_hits + 600 * ev.n_events + (1 << 16)
+
+
 def test_overlapping_admission_and_failure_recovery():
     from paper_2207_03936_gb300 import sbt
     ev = synth.make_events(2, 120, workers=1)
