@@ -927,7 +927,13 @@ __device__ bool search_stage(const DevConfig& C, const Region<HS>& R, const Smem
         // P1
         int na = 0, nc = -1, nb = 0;  // this lane's new seed
         int i0 = (tid >> 5) * kSeedGroups, batch = 0;
-        for (;;) {
+        // A warp without middle hits is needed only if the old tracks fill the
+        // warps before it that have none.  Otherwise its one round finds nothing
+        // and still takes the issue slots of the other blocks' warps: search of
+        // 200000 events of 20 hits 7.42 -> 6.25 ms, of 5000 events of 686 hits
+        // 549 -> 547 us, of 500 events of 4200 hits 408 us either way.
+        const int rank = (tid >> 5) - (nl + kSeedGroups - 1) / kSeedGroups;
+        while (i0 < nl || (follow && nold > 32 * rank)) {
             if (i0 < nl) {
                 const int i = i0 + lane / kSeedLanes;
                 const uint32_t mk = i < nl ? list[i] : 0u;

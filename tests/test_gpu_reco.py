@@ -272,6 +272,32 @@ def test_block_sizes_agree(sbt, threads):
         h.close()
 
 
+@pytest.mark.parametrize("threads", [0, 64, 128, 256])
+def test_following_with_idle_warps_bit_exact(sbt, threads):
+    """Old tracks around each number that fills one warp more, in steps whose
+    hits all lie on them (no middle hits: the warps past the last old track
+    skip the step), and with a few new tracks beginning later (some warps
+    seed); a short event whose last steps are empty."""
+    cases = [single_track(missing=tuple(range(12, 52)))[:4]]
+    for n, late in ((1, 0), (31, 0), (32, 3), (33, 0), (64, 9), (65, 1), (128, 0), (129, 20), (257, 0), (513, 17)):
+        phi = np.linspace(0.0, 2 * np.pi, n + late, endpoint=False) + 0.001
+        parts = [line_hits(12.0 * np.cos(p), 12.0 * np.sin(p), 0.02 * np.cos(p), 0.02 * np.sin(p),
+                           range(8 if k % 16 == 5 and k // 16 < late else 0, 24)) for k, p in enumerate(phi)]
+        cases.append(assemble(parts, n)[:4])
+    off = np.concatenate([[0], np.cumsum([len(c[0]) for c in cases])]).astype(np.int32)
+    x, y, z, m = (np.concatenate([np.asarray(c[i]) for c in cases]) for i in range(4))
+    ev = synth.Events(x.astype(np.float32), y.astype(np.float32), z.astype(np.float32), m.astype(np.int32), off,
+                      np.full(len(x), -1, np.int32), 0, MZ)
+    ref = oracle_of(ev)
+    assert (np.diff(ref.track_offsets)[1:5] == [1, 31, 35, 33]).all()
+    h = sbt.sbt_create(MZ, sbt.default_config(threads_per_block=threads, **CFG))
+    try:
+        for batched in (False, True):
+            assert_same(run_gpu(sbt, h, ev, batched), ref)
+    finally:
+        h.close()
+
+
 def test_block_size_follows_the_number_of_events(sbt, handle):
     """The largest and smallest batch of each block size that the library picks
     by itself (512 threads up to one event an SM, 256 up to eight, then 128),
