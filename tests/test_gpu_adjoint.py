@@ -184,6 +184,28 @@ def test_adjoint_long_tracks_that_share_modules(setup, per_module):
     assert torch.equal(c, c2) and torch.equal(g, g2)
 
 
+@pytest.mark.parametrize("lengths", [[3], [2, 1, 0], [65, 64, 2, 63], [20, 24, 17, 33], [200, 3, 5], [160]],
+                         ids=lambda v: "-".join(map(str, v)))
+@pytest.mark.parametrize("n_tracks", [0, 1, 31, 129, 2000])
+def test_adjoint_value_only(setup, n_tracks, lengths):
+    """A call without a gradient leaves out forces, torques and their order by
+    module: the value and the skipped count stay those of the full call, bit
+    for bit, with invalid tracks among them."""
+    sbt, h, ev, _, _, d = setup
+    rng = np.random.default_rng([n_tracks, *lengths])
+    ho = np.concatenate([[0], np.cumsum(np.resize(np.array(lengths), n_tracks))]).astype(np.int32)
+    th = rng.integers(0, ev.n_hits, int(ho[-1])).astype(np.int32)
+    if n_tracks > 100 and len(th) > 500:
+        th[len(th) // 2] = ev.n_hits
+    align = np.concatenate([rng.normal(0, 0.005, (52, 3)), rng.normal(0, 5e-5, (52, 3))], 1)
+    args = [d["x"], d["y"], d["z"], d["m"], torch.from_numpy(ho).cuda(), torch.from_numpy(th).cuda(),
+            torch.from_numpy(align).cuda()]
+    c, g, sk = sbt.sbt_fit_adjoint(h, *args, with_skipped=True)
+    c2, none, sk2 = sbt.sbt_fit_adjoint(h, *args, want_grad=False, with_skipped=True)
+    assert none is None and g.shape == (52, 6)
+    assert torch.equal(c, c2) and torch.equal(sk, sk2)
+
+
 @pytest.mark.parametrize("value", [3e38, np.inf, np.nan], ids=str)
 def test_adjoint_beyond_fp32_sums(setup, value):
     """Positions whose fp32 sum overflows keep the fp64 result; infinities and
