@@ -294,6 +294,10 @@ sbt_status sbt_reconstruct_noalloc(sbt_handle* h, const float* x, const float* y
  * accounting for benchmarks); 0 before any call. */
 int32_t sbt_last_launch_count(const sbt_handle* h);
 
+/* Threads of a search block in the last reconstruction call on h: the configured
+ * or tuned number, else by the number of events; 0 before any call. */
+int32_t sbt_last_block_threads(const sbt_handle* h);
+
 /* Number of graphs sbt_reconstruct_batched has captured on h: a call with new
  * arrays, sizes or launch shape captures one, and so does the first call after
  * another entry point has replaced a workspace of h. */
@@ -378,6 +382,10 @@ sbt_status sbt_server_release(sbt_server* s, int64_t request_id);
  * batch they meet and then allocate nothing; buffers they outgrow are kept
  * until sbt_server_destroy, since freeing would stall the device). */
 sbt_status sbt_server_stats(sbt_server* s, double* stats);
+
+/* Threads of a search block in the last batch launched (by its events times the
+ * slots, which share the GPU); 0 before any batch. */
+int32_t sbt_server_block_threads(const sbt_server* s);
 
 /* Makes the next launched batch fail on the host side (test hook for the
  * failure path: the batch's requests complete with SBT_ERR_CUDA status and

@@ -173,6 +173,7 @@ struct sbt_handle {
     bool have_key = false;
     int captures = 0;  // graphs captured so far
     int launches_last = 0;
+    int threads_last = 0;  // of a search block
 };
 
 namespace {
@@ -329,7 +330,11 @@ void handle_set_serving(sbt_handle* h, int slots)
 
 void handle_set_error(sbt_handle* h, const std::string& msg) { h->err = msg; }
 
-void handle_set_launches(sbt_handle* h, int launches) { h->launches_last = launches; }
+void handle_set_launches(sbt_handle* h, int launches, int threads)
+{
+    h->launches_last = launches;
+    h->threads_last = threads;
+}
 
 void handle_defer_frees(sbt_handle* h)
 {
@@ -469,10 +474,11 @@ sbt_status sbt_reconstruct(sbt_handle* h, const float* x, const float* y, const 
     carve_work(h->plain_arena.base, n_hits, n_events, &W);
     Inputs in = make_inputs(x, y, z, module, event_offsets, n_events, n_hits);
     e = launch_sort(h->C, in, O, s);
-    if (e == cudaSuccess) e = launch_plain(h->C, in, O, W, S, *out, default_threads(h, false, n_events), s);
+    const int threads = default_threads(h, false, n_events);
+    if (e == cudaSuccess) e = launch_plain(h->C, in, O, W, S, *out, threads, s);
     if (e == cudaSuccess) e = launch_finish(h->C, in, S, *out, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "plain launch");
-    h->launches_last = n_events > 0 ? 2 + finish_launches(n_events) : 2;
+    handle_set_launches(h, n_events > 0 ? 2 + finish_launches(n_events) : 2, threads);
     return SBT_OK;
 }
 
@@ -535,7 +541,7 @@ sbt_status sbt_reconstruct_batched(sbt_handle* h, const float* x, const float* y
     }
     cudaError_t e = cudaGraphLaunch(h->exec, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "graph launch");
-    h->launches_last = n_events > 0 ? 3 + finish_launches(n_events) : 2;
+    handle_set_launches(h, n_events > 0 ? 3 + finish_launches(n_events) : 2, threads);
     return SBT_OK;
 }
 
@@ -745,7 +751,7 @@ sbt_status sbt_reconstruct_host(sbt_handle* h, const float* x, const float* y, c
     oh->counts[1] = (int32_t)HH;
     oh->counts[2] = cap_ok ? SBT_OK : SBT_ERR_CAPACITY;
     oh->counts[3] = (int32_t)failed;
-    h->launches_last = C > 1 || n_events == 0 ? C * 7 : 4 + finish_launches(n_events);
+    handle_set_launches(h, C > 1 || n_events == 0 ? C * 7 : 4 + finish_launches(n_events), threads);
     return SBT_OK;
 }
 
@@ -953,6 +959,9 @@ sbt_status sbt_profile_batched(sbt_handle* h, const float* x, const float* y, co
 
 /* Number of kernels the last reconstruction call enqueued (for launch accounting). */
 int32_t sbt_last_launch_count(const sbt_handle* h) { return h ? h->launches_last : 0; }
+
+/* Threads of a search block in the last reconstruction call. */
+int32_t sbt_last_block_threads(const sbt_handle* h) { return h ? h->threads_last : 0; }
 
 /* Number of graphs sbt_reconstruct_batched has captured on the handle. */
 int32_t sbt_graph_captures(const sbt_handle* h) { return h ? h->captures : 0; }

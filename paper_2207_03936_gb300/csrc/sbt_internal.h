@@ -198,7 +198,7 @@ Tables handle_tables(const sbt_handle* h, int64_t n_events);
 // counts them.
 void handle_set_serving(sbt_handle* h, int slots);
 void handle_set_error(sbt_handle* h, const std::string& msg);
-void handle_set_launches(sbt_handle* h, int launches);
+void handle_set_launches(sbt_handle* h, int launches, int threads);
 // Workspaces the handle outgrows are kept until sbt_destroy instead of freed
 // (cudaFree synchronises the device); for handles whose work overlaps other
 // streams' work, such as the serving slots.

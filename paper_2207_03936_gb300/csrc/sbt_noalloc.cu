@@ -181,12 +181,13 @@ extern "C" sbt_status sbt_reconstruct_noalloc(sbt_handle* h, const float* x, con
     cudaStream_t s = (cudaStream_t)stream;
     const DevConfig& C = handle_device_config(h);
     e = launch_sort(C, in, O, s);
-    if (e == cudaSuccess) e = launch_plain(C, in, O, W, S, *out, handle_plain_threads(h, n_events), s);
+    const int threads = handle_plain_threads(h, n_events);
+    if (e == cudaSuccess) e = launch_plain(C, in, O, W, S, *out, threads, s);
     if (e == cudaSuccess) e = launch_finish(C, in, S, *out, s);
     if (e != cudaSuccess) {
         handle_set_error(h, std::string("noalloc launch: ") + cudaGetErrorString(e));
         return SBT_ERR_CUDA;
     }
-    handle_set_launches(h, n_events > 0 ? 2 + finish_launches(n_events) : 2);
+    handle_set_launches(h, n_events > 0 ? 2 + finish_launches(n_events) : 2, threads);
     return SBT_OK;
 }

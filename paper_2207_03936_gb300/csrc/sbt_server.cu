@@ -224,6 +224,7 @@ struct sbt_server {
     // per-batch time sums (ms): uploads, kernels, downloads on the slot's
     // stream (CUDA events), and enqueue to harvest on the host clock
     double st_up_ms = 0, st_kern_ms = 0, st_down_ms = 0, st_wall_ms = 0, st_timed = 0;
+    std::atomic<int32_t> block_threads{0};  // of a search block in the last batch
     std::atomic<double> st_launch_s{0.0};  // launcher time spent enqueueing batches
     int64_t allocs0 = 0;                    // g_allocs when the server was created
     std::thread launcher, harvester, feeder;
@@ -382,6 +383,7 @@ void launcher_loop(sbt_server* S)
             cudaStreamSynchronize(sl.stream);  // drain what was enqueued before reuse
             sl.failed = true;
         }
+        if (!sl.failed) S->block_threads.store(sbt_last_block_threads(sl.h), std::memory_order_relaxed);
         S->st_launch_s.store(S->st_launch_s.load(std::memory_order_relaxed) + (now_s() - tl),
                              std::memory_order_relaxed);
         sl.busy.store(true, std::memory_order_release);
@@ -764,6 +766,11 @@ sbt_status sbt_server_stats(sbt_server* S, double* stats)
     stats[12] = S->st_timed;
     stats[13] = (double)(g_allocs.load() - S->allocs0);
     return SBT_OK;
+}
+
+int32_t sbt_server_block_threads(const sbt_server* S)
+{
+    return S ? S->block_threads.load(std::memory_order_relaxed) : 0;
 }
 
 sbt_status sbt_server_inject_failure(sbt_server* S)

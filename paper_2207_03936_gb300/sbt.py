@@ -83,6 +83,7 @@ def lib() -> ctypes.CDLL:
             "sbt_debug_sort": (_I32, [_P, _P, _P, _P, _P, _I32, _I32, _P, _P, _P, _P]),
             "sbt_debug_phi16": (_I32, [_P, _P, _I32, _P, _P]),
             "sbt_last_launch_count": (_I32, [_P]),
+            "sbt_last_block_threads": (_I32, [_P]),
             "sbt_graph_captures": (_I32, [_P]),
             "sbt_profile_batched": (_I32, [_P, _P, _P, _P, _P, _P, _I32, _I32, _P, _I32, _P, _P]),
         }
@@ -216,6 +217,9 @@ class Handle:
 
     def last_launch_count(self) -> int:
         return int(lib().sbt_last_launch_count(self.h))
+
+    def last_block_threads(self) -> int:
+        return int(lib().sbt_last_block_threads(self.h))
 
     def graph_captures(self) -> int:
         return int(lib().sbt_graph_captures(self.h))
@@ -393,6 +397,7 @@ def _server_sigs():
         "sbt_server_drain": (_I32, [_P, _P, _P, _P, _I32, _P, ctypes.c_double]),
         "sbt_server_release": (_I32, [_P, _I64]),
         "sbt_server_stats": (_I32, [_P, _P]),
+        "sbt_server_block_threads": (_I32, [_P]),
         "sbt_server_inject_failure": (_I32, [_P]),
         "sbt_server_destroy": (_I32, [_P]),
     }
@@ -489,6 +494,9 @@ class Server:
                 "peak_bytes": v[4], "failed_batches": v[5], "feed_lag_s": v[6],
                 "launch_busy_s": v[7], "upload_ms": v[8], "kernel_ms": v[9], "download_ms": v[10],
                 "batch_wall_ms": v[11], "timed_batches": v[12], "allocations": v[13]}
+
+    def block_threads(self) -> int:
+        return int(self.L.sbt_server_block_threads(self.s))
 
     def inject_failure(self):
         _check(self.L.sbt_server_inject_failure(self.s))

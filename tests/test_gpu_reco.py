@@ -228,12 +228,18 @@ def test_global_event_cut(sbt, batched):
     assert np.array_equal(g["chi2"].view(np.uint32), want["chi2"].view(np.uint32))
 
 
+# Block sizes of the tests below: the one the library picks for their batches,
+# mostly 512, and those that larger batches run.
+BLOCKS = pytest.mark.parametrize("threads", [0, 128, 256])
+
+
+@BLOCKS
 @pytest.mark.parametrize("config,n", [(2, 300), (3, 150)])
-def test_fp16_hit_storage_bit_exact(sbt, config, n):
+def test_fp16_hit_storage_bit_exact(sbt, config, n, threads):
     """fp16 hit storage: plain and batched equal the oracle run on coordinates
     rounded to fp16; the sort stage equals the oracle's sort of them."""
     ev = synth.make_events(config, n)
-    h = sbt.sbt_create(ev.module_z, sbt.default_config(fp16_hits=1, **CFG))
+    h = sbt.sbt_create(ev.module_z, sbt.default_config(fp16_hits=1, threads_per_block=threads, **CFG))
     try:
         o = oracle.reconstruct(ev.x, ev.y, ev.z, ev.module, ev.event_offsets, ev.module_z,
                                oracle.config(**CFG), fp16_hits=True)
@@ -305,17 +311,19 @@ def test_block_size_follows_the_number_of_events(sbt, handle):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     ev = synth.make_events(1, 8 * sms + 1, workers=1)
     ref = oracle_of(ev)
-    for e in (1, sms, sms + 1, 8 * sms, 8 * sms + 1):
+    for e, threads in ((1, 512), (sms, 512), (sms + 1, 256), (8 * sms, 256), (8 * sms + 1, 128)):
         t = int(ref.track_offsets[e])
         hits = int(ref.hit_offsets[t])
         for batched in (False, True):
             g = run_gpu(sbt, handle, ev.subset(0, e), batched)
+            assert handle.last_block_threads() == threads
             assert np.array_equal(g["track_offsets"], ref.track_offsets[:e + 1])
             assert np.array_equal(g["track_hits"], ref.track_hits[:hits])
             assert np.array_equal(g["params"].view(np.uint32), ref.params[:t].view(np.uint32))
 
 
-def test_hand_built_events(sbt, handle):
+@BLOCKS
+def test_hand_built_events(sbt, threads):
     cases = []
     x, y, z, m, _ = single_track()
     cases.append((x, y, z, m))
@@ -344,8 +352,12 @@ def test_hand_built_events(sbt, handle):
                       np.concatenate(ms).astype(np.int32), np.array(offs, np.int32),
                       np.zeros(offs[-1], np.int32), 0, MZ)
     o = oracle_of(ev)
-    assert_same(run_gpu(sbt, handle, ev, False), o)
-    assert_same(run_gpu(sbt, handle, ev, True), o)
+    h = sbt.sbt_create(MZ, sbt.default_config(threads_per_block=threads, **CFG))
+    try:
+        assert_same(run_gpu(sbt, h, ev, False), o)
+        assert_same(run_gpu(sbt, h, ev, True), o)
+    finally:
+        h.close()
 
 
 def test_edge_cases_empty_and_degenerate(sbt, handle):
@@ -648,8 +660,9 @@ def test_autotune_keeps_results(sbt):
         h.close()
 
 
+@BLOCKS
 @pytest.mark.parametrize("fp16", [0, 1])
-def test_maximum_event_size_bit_exact(sbt, fp16):
+def test_maximum_event_size_bit_exact(sbt, fp16, threads):
     """An event of exactly the largest supported size (16384 hits: the sort's
     shared-memory buffers and the 16-bit hit positions of the search) between
     two ordinary events, through the plain, batched and host entry points; an
@@ -664,7 +677,8 @@ def test_maximum_event_size_bit_exact(sbt, fp16):
     offs = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int32)
     ev = synth.Events(cat(base.x), cat(base.y), cat(base.z), cat(base.module), offs,
                       cat(base.mc), 0, base.module_z)
-    h = sbt.sbt_create(ev.module_z, sbt.default_config(max_hits_per_event=16384, fp16_hits=fp16, **CFG))
+    h = sbt.sbt_create(ev.module_z, sbt.default_config(max_hits_per_event=16384, fp16_hits=fp16, threads_per_block=threads,
+                                                       **CFG))
     try:
         ref = oracle.reconstruct(ev.x, ev.y, ev.z, ev.module, ev.event_offsets, ev.module_z,
                                  oracle.config(**CFG), fp16_hits=bool(fp16))
@@ -690,13 +704,15 @@ def test_maximum_event_size_bit_exact(sbt, fp16):
         h.close()
 
 
+@BLOCKS
 @pytest.mark.parametrize("config,n,fp16", [(2, 150, 0), (3, 60, 0), (2, 80, 1)])
-def test_module_pairs_bit_exact(sbt, config, n, fp16):
+def test_module_pairs_bit_exact(sbt, config, n, fp16, threads):
     """Module-pair geometry (two one-sided planes per module, the x < 0 plane
     at module_z2): plain, batched and host entry points equal the oracle's
     pair reading, fp32 and fp16 storage."""
     ev = synth.make_events(config, n, pairs=True)
-    h = sbt.sbt_create(ev.module_z, sbt.default_config(fp16_hits=fp16, **CFG), module_z2=ev.module_z2)
+    h = sbt.sbt_create(ev.module_z, sbt.default_config(fp16_hits=fp16, threads_per_block=threads, **CFG),
+                       module_z2=ev.module_z2)
     try:
         o = oracle.reconstruct(ev.x, ev.y, ev.z, ev.module, ev.event_offsets, ev.module_z,
                                oracle.config(**CFG), fp16_hits=bool(fp16), module_z2=ev.module_z2)
@@ -732,8 +748,9 @@ def test_module_pairs_adjoint_is_refused(sbt):
         h.close()
 
 
+@BLOCKS
 @pytest.mark.parametrize("cfg_seed", range(4))
-def test_crowded_tiny_events_bit_exact(sbt, cfg_seed):
+def test_crowded_tiny_events_bit_exact(sbt, cfg_seed, threads):
     # the crowded tiny events of the oracle's whole-loop pin (overlapping
     # seeds, contended extensions, overlapping tracklets), 200 per batch on
     # eight planes, under four random configurations
@@ -748,7 +765,7 @@ def test_crowded_tiny_events_bit_exact(sbt, cfg_seed):
                       np.zeros(offs[-1], np.int32), 0, module_z)
     o = oracle.reconstruct(ev.x, ev.y, ev.z, ev.module, ev.event_offsets, module_z, oracle.config(**cfg))
     assert o.n_tracks > 200
-    h = sbt.sbt_create(module_z, sbt.default_config(**cfg))
+    h = sbt.sbt_create(module_z, sbt.default_config(threads_per_block=threads, **cfg))
     try:
         for batched in (False, True):
             assert_same(run_gpu(sbt, h, ev, batched), o)
@@ -756,9 +773,10 @@ def test_crowded_tiny_events_bit_exact(sbt, cfg_seed):
         h.close()
 
 
+@BLOCKS
 @pytest.mark.parametrize("per_module", [1, 2, 31, 33, 100])
 @pytest.mark.parametrize("k", [1, 4, 5, 9])
-def test_candidate_lanes_and_bucket_windows_bit_exact(sbt, k, per_module):
+def test_candidate_lanes_and_bucket_windows_bit_exact(sbt, k, per_module, threads):
     """Seeding's lanes (K below, at and above the four lanes of a middle hit;
     fewer outer hits than K; more middle hits than a warp's eight groups) and
     the window scans from the bucket table (hits around phi = +-pi, where a
@@ -780,7 +798,7 @@ def test_candidate_lanes_and_bucket_windows_bit_exact(sbt, k, per_module):
     cut = 0.3 if per_module < 64 else 0.02
     cfg = dict(CFG, k_doublets=k, max_scatter_seed=cut, max_scatter_follow=0.2, max_chi2_tracklet=5000.0)
     ref = oracle.reconstruct(ev.x, ev.y, ev.z, ev.module, ev.event_offsets, ev.module_z, oracle.config(**cfg))
-    h = sbt.sbt_create(ev.module_z, sbt.default_config(**cfg))
+    h = sbt.sbt_create(ev.module_z, sbt.default_config(threads_per_block=threads, **cfg))
     try:
         for batched in (False, True):
             assert_same(run_gpu(sbt, h, ev, batched), ref)

@@ -50,6 +50,28 @@ def test_served_results_equal_results_alone():
         assert r.latency_s > 0
 
 
+@pytest.mark.parametrize("slots,events", [(1, 1), (1, 200), (4, 30), (4, 50), (4, 400)])
+def test_served_block_size_follows_events_and_slots(slots, events):
+    """A batch's block size goes by its events times the slots, which share the
+    GPU: 512 threads up to one event an SM, 256 up to eight, then 128."""
+    from paper_2207_03936_gb300 import sbt
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ev = synth.make_events(1, events, workers=1)
+    h = sbt.sbt_create(ev.module_z, sbt.default_config())
+    srv = sbt.Server(h, memory_budget_bytes=1 << 30, max_streams=slots, max_batch_events=events)
+    try:
+        srv.submit_schedule(ev, np.zeros(ev.n_events))
+        got = collect(srv, ev.n_events)
+        st = srv.stats()
+        threads = srv.block_threads()
+    finally:
+        srv.close()
+        h.close()
+    assert len(got) == events and st["batches"] == 1
+    shared = slots * events
+    assert threads == (512 if shared <= sms else 256 if shared <= 8 * sms else 128)
+
+
 def test_admission_counts_the_hits_of_quiet_events():
     """The bytes a batch counts against the budget follow its hits (112 a hit and
     600 an event at 52 modules), also for events of a few hundred hits."""
