@@ -194,11 +194,11 @@ sbt_status cuda_fail(sbt_handle* h, cudaError_t e, const char* where)
 // block on the GPU at once, the call takes as long as the steps of its largest
 // event, and more warps shorten a step; beyond that the resident events count.
 // Two blocks of 512 fit an SM (64 registers), eight of 256, sixteen of 128 (32
-// registers).  Search, us at 512 / 256 / 128 threads: one event 230 / 251 /
-// 263, 100 events 336 / 402 / 574, 500 events 481 / 426 / 600, 1000 events
-// 960 / 531 / 693, 16000 events - / 6376 / 5397.  512 only up to one event an
-// SM, so that calls on several streams still run side by side: 300 events a
-// call on eight streams make 1.09, 1.94 and 1.88 M events/s.
+// registers).  Search, us at 512 / 256 / 128 threads: one event 200 / 226 /
+// 246, 100 events 284 / 372 / 510, 500 events 431 / 408 / 556, 1000 events
+// 866 / 498 / 659, 16000 events 13688 / 5856 / 4993.  512 only up to one event
+// an SM, so that calls on several streams still run side by side: 300 events a
+// call on eight streams make 1.09, 1.94 and 1.87 M events/s.
 int default_threads(const sbt_handle* h, bool batched, int64_t n_events)
 {
     if (h->cfg.threads_per_block) return h->cfg.threads_per_block;

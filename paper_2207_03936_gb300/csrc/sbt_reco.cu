@@ -101,9 +101,9 @@ __device__ __forceinline__ float scatter_of(float4 B, float xp, float yp)
 }
 
 // Least-squares straight line through n hits (get(i) -> float3 in hit
-// order): params (x0, y0, tx, ty) at z = 0 and chi2 = residual sum / sigma^2.
+// order): chi2 = residual sum / sigma^2.
 template <class Get>
-__device__ __forceinline__ void fit_line(int n, Get get, float sigma, float* params, float* chi2)
+__device__ __forceinline__ float fit_chi2(int n, Get get, float sigma)
 {
     float nf = (float)n;
     float sx = 0.0f, sy = 0.0f, sz = 0.0f;
@@ -132,13 +132,7 @@ __device__ __forceinline__ void fit_line(int n, Get get, float sigma, float* par
         float ry = __fsub_rn(__fsub_rn(h.y, ym), __fmul_rn(ty, dz));
         s = __fadd_rn(s, __fadd_rn(__fmul_rn(rx, rx), __fmul_rn(ry, ry)));
     }
-    if (params) {
-        params[0] = __fsub_rn(xm, __fmul_rn(tx, zm));
-        params[1] = __fsub_rn(ym, __fmul_rn(ty, zm));
-        params[2] = tx;
-        params[3] = ty;
-    }
-    *chi2 = __fdiv_rn(s, __fmul_rn(sigma, sigma));
+    return __fdiv_rn(s, __fmul_rn(sigma, sigma));
 }
 
 // ------------------------------------------------------- shared layout ---
@@ -1061,14 +1055,13 @@ __device__ void tracklet_filter(const DevConfig& C, const Region<HS>& R, const S
         int key = (int)(v >> 48);
         uint32_t q = 0xFFFFFFFFu;
         if (!flagged(S, h[0]) && !flagged(S, h[1]) && !flagged(S, h[2])) {
-            float chi2;
-            fit_line(
+            const float chi2 = fit_chi2(
                 3,
                 [&](int i) {
                     float4 c = R.coords[h[i]];
                     return make_float3(c.x, c.y, c.z);
                 },
-                C.sigma, nullptr, &chi2);
+                C.sigma);
             if (chi2 < C.C3) {
                 q = __float_as_uint(chi2);
                 unsigned long long kk = claim_key(0ull, chi2, key);
@@ -1201,9 +1194,10 @@ __device__ void run_event(const DevConfig& C, const Inputs& in, const Sorted& O,
 // Residency of the search: the kernel waits on load latency, so throughput
 // follows the number of resident events; the compiler is asked for a
 // register count that lets 2048 threads share an SM (16 blocks of 128, 16000
-// uneven events: 5.40 ms; 1536 threads 5.94, 1024 threads 6.65).  Blocks of 512
+// uneven events: 4.99 ms; 1536 threads 5.34, 1024 threads 6.07).  Blocks of 512
 // run calls of a few events, where a step's length counts: 64 registers, no
-// spills (one event 251 us at 256 threads and 32 registers, 229 us at 64).
+// spills (one event 226 us at 256 threads and 32 registers, 204 at 64; 200 us at
+// 512).
 constexpr int search_blocks_per_sm(int threads) { return (threads == 512 ? 1024 : 2048) / threads; }
 
 // One block per event.
@@ -1403,7 +1397,7 @@ __global__ void __launch_bounds__(kOutputThreads) k_output(DevConfig C, Inputs i
 // without conflicts (33 words a row).  With each lane
 // loading its own track's records and storing its own hit list, every lane was
 // an L1 wavefront of its own (two a hit, the LSU data pipe 74% busy).  The sums
-// run in hit order, every operation rounded as in fit_line.
+// run in hit order, every operation rounded as in fit_chi2.
 constexpr int kFitThreads = 128;
 constexpr int kFitRows = 16;
 constexpr int kFitAhead = 4;
