@@ -388,7 +388,8 @@ k_adjoint(DevConfig C, Inputs in, const int32_t* hit_offsets, const int32_t* tra
             // line), so the fp64 pipe takes no sums of positions, and the means
             // carry the rounding of micrometres instead of that of metres.
             // Gradient error against 128-bit sums, over that of a tree of sums:
-            // 0.92 / 0.94 / 0.98 / 0.99 at 1 / 8 / 60 / 400 events; sums of
+            // 0.92 / 0.94 / 0.98 / 0.99 at 1 / 8 / 60 / 400 events, 1.00 at 2000
+            // and 10000 (the rounding of the rotations, common to both); sums of
             // positions in fp64, by fours, 1.09 / 1.07 / 1.03 / 1.01 (10000
             // events 5154 us, here 5363), their means corrected by the sums of
             // differences 0.92 / 0.93 / 0.98 / 0.99 (5517 us).
