@@ -141,6 +141,7 @@ enum Misc {
     kErr = 0, kNFin = 1, kNTl = 2, kEvent = 3, kCMask = 4, kCnt0 = 5, kCnt1 = 6, kWork = 7, kNew = 8, kList = 9,
     kNOuter = 10, kShift = 11, kMiscN = 12
 };
+static_assert(kMiscN % 2 == 0, "a pointer follows");
 
 // Per-block shared memory of the search: flag bits, module offsets, counters,
 // each sized to what the configuration needs.  Everything sized by the event
@@ -151,13 +152,17 @@ struct Smem {
     uint32_t* flag;     // one bit per sorted position
     int* modoff;
     int* misc;
+    // first sorted position of each (module, phi16 >> misc[kShift]); here and not
+    // in registers, which the windows are short of (calls of 16 quiet events 155
+    // -> 153 us, 100 events 338 -> 334, 500 events 482 -> 477)
+    const uint16_t** table;
     int* wsum;          // [33]
 };
 
 __host__ __device__ inline size_t align16(size_t v) { return (v + 15) & ~(size_t)15; }
 
 struct Plan {
-    size_t flag, modoff, misc, wsum, total;
+    size_t flag, modoff, misc, table, wsum, total;
 };
 
 __host__ __device__ inline Plan make_plan(int nmax, int threads, int M)
@@ -166,7 +171,8 @@ __host__ __device__ inline Plan make_plan(int nmax, int threads, int M)
     size_t o = 0;
     p.flag = o;     o = align16(o + 4 * (((size_t)nmax + 31) / 32));
     p.modoff = o;   o = align16(o + 4 * ((size_t)M + 1));
-    p.misc = o;     o = align16(o + 4 * kMiscN);
+    p.misc = o;     o = o + 4 * kMiscN;
+    p.table = o;    o = align16(o + sizeof(void*));
     p.wsum = o;     o = align16(o + 4 * ((size_t)threads / 32 + 1));
     p.total = o;
     return p;
@@ -181,6 +187,7 @@ __device__ inline Smem carve(unsigned char* raw, int nmax, int threads, int M)
     S.flag = (uint32_t*)(raw + p.flag);
     S.modoff = (int*)(raw + p.modoff);
     S.misc = (int*)(raw + p.misc);
+    S.table = (const uint16_t**)(raw + p.table);
     S.wsum = (int*)(raw + p.wsum);
     return S;
 }
@@ -243,7 +250,6 @@ struct HitArr {
 template <class HS>
 struct Region {
     HitArr<HS> coords;
-    const uint16_t* bucket;     // first sorted position of each (module, phi16 >> misc[kShift])
     uint32_t* list;
     uint16_t* prev;
     unsigned long long* claim;  // the search's claim of sorted position p is claim[p & cmask]
@@ -258,12 +264,10 @@ struct Region {
 };
 
 template <class HS>
-__device__ inline Region<HS> region_of(const Sorted& O, int M, int e, int off, const Work& W, int64_t hb,
-                                      int64_t r, int cap)
+__device__ inline Region<HS> region_of(const Sorted& O, int off, const Work& W, int64_t hb, int64_t r, int cap)
 {
     Region<HS> R;
     R.coords = HitArr<HS>{(const typename HS::T*)O.coords + off, O.index + off};
-    R.bucket = O.bucket + table_base(O.tables, off, e);
     R.list = W.list + hb;
     R.prev = W.prev + hb;
     R.claim_all = W.claim + hb;
@@ -658,8 +662,7 @@ __device__ __forceinline__ unsigned long long best_hit(const DevConfig& C, const
             if (window_of(xp, yp, cut, sqrt_cut, lo, width)) {
                 const int shift = S.misc[kShift];
                 const uint32_t k = (uint32_t)bucket_of(t, lo, shift);
-                b = R.bucket[k];
-                b = max(b, b0);
+                b = max((*S.table)[k], b0);
                 b = b < b1 ? b : b0;
                 const uint32_t edge = k << shift << 16;  // the bucket's, above the low bits
                 width = ((width + lo) << 16 | 0xFFFFu) - edge;
@@ -1154,7 +1157,7 @@ __device__ void run_event(const DevConfig& C, const Inputs& in, const Sorted& O,
         fail_event(e, st != SBT_OK ? st : SBT_ERR_CAPACITY, G, out);
         return;
     }
-    Region<HS> R = region_of<HS>(O, C.M, e, off, W, hb, r, cap);
+    Region<HS> R = region_of<HS>(O, off, W, hb, r, cap);
     for (int m = tid; m <= C.M; m += NT) S.modoff[m] = O.modoff[(int64_t)e * (C.M + 1) + m];
     for (int w = tid; w < (n + 31) / 32; w += NT) S.flag[w] = 0u;
     __syncthreads();
@@ -1170,7 +1173,10 @@ __device__ void run_event(const DevConfig& C, const Inputs& in, const Sorted& O,
         w = __reduce_max_sync(0xFFFFFFFFu, w);
         const int p2 = w > 1 ? 1 << (32 - __clz(w - 1)) : 1;
         if (tid == 0) S.misc[kCMask] = p2 <= cap ? p2 - 1 : -1;
-        if (tid == 0) S.misc[kShift] = 16 - bucket_bits(O.tables, n, C.M);
+        if (tid == 0) {
+            S.misc[kShift] = 16 - bucket_bits(O.tables, n, C.M);
+            *S.table = O.bucket + table_base(O.tables, off, e);
+        }
         if (tid < kMiscN && tid != kCMask && tid != kEvent && tid != kShift) S.misc[tid] = 0;
     }
     __syncthreads();
